@@ -244,6 +244,10 @@ struct Launch {
   static void apply_bwd(const ApplyRec* recs, const int* ids, int nids, int maxm, int maxnw,
                         const real* fac, const int64_t* vmap, real* y, real* z, real* part,
                         int64_t ldy, int nrhs, cudaStream_t st);
+  // both sweeps of a level that is one dense cluster of n unknowns without
+  // neighbours (the last level): z = T' y, y = T_R'^T z
+  static void apply_top(const ApplyRec* recs, const int* ids, int n, bool sym, const real* fac,
+                        real* y, real* z, int64_t ldy, int nrhs, cudaStream_t st);
   static void scatter_csr(const int64_t* dst, const double* val, int64_t nnz, real* arena,
                           cudaStream_t st);
   static void gather_vec(const int64_t* idx, int64_t n, const real* src, int64_t lds,

@@ -1593,6 +1593,14 @@ struct LevelVecs {
   void* part;
 };
 
+// The dense top as the sweeps see it: the last level, one cluster, large
+// enough that its triangular operators are streamed by kernels of their own
+// (up to kTopOneCta unknowns one CTA cluster holds them in shared memory).
+bool apply_as_top(const FLevel& F) {
+  return F.top && F.cls.size() == 1 && F.cls[0].size() == 1 && F.cls_maxm[0] > kTopOneCta &&
+         F.cls_maxnw[0] == 0 && F.k[0] == 0;
+}
+
 // The level sweeps of Alg. 2 between the level-0 vector and itself: a fixed
 // sequence of launches once the factorization and nrhs are fixed (one group
 // of launches per colour class and direction).
@@ -1603,6 +1611,12 @@ void apply_levels(hsolve_handle* h, int nrhs, cudaStream_t st, const std::vector
   for (int l = 0; l < L; l++) {
     FLevel& F = *h->F[l];
     const int64_t nl = std::max<int64_t>(F.P.voff[F.P.nclu], 1);
+    if (l + 1 == L && apply_as_top(F)) {
+      Launch<real>::apply_top(F.recs.as<ApplyRec>(), F.ids.as<int>(), F.cls_maxm[0],
+                              h->symmetric != 0, F.fac.as<real>(), vec(l),
+                              static_cast<real*>(B[l].zvec), nl, nrhs, st);
+      continue;
+    }
     for (size_t c = 0; c < F.cls.size(); c++)
       Launch<real>::apply_fwd(F.recs.as<ApplyRec>(), F.ids.as<int>() + F.cls_off[c],
                               (int)F.cls[c].size(), F.cls_maxm[c], F.cls_maxnw[c],
@@ -1624,6 +1638,7 @@ void apply_levels(hsolve_handle* h, int nrhs, cudaStream_t st, const std::vector
       Launch<real>::scatter_vec(F.next_idx.as<int64_t>(), F.next_n, vec(l + 1), ng, vec(l), nl,
                                 nrhs, st);
     }
+    if (l + 1 == L && apply_as_top(F)) continue;  // both sweeps ran above
     for (int c = (int)F.cls.size() - 1; c >= 0; c--)
       Launch<real>::apply_bwd(F.recs.as<ApplyRec>(), F.ids.as<int>() + F.cls_off[c],
                               (int)F.cls[c].size(), F.cls_maxm[c], F.cls_maxnw[c],

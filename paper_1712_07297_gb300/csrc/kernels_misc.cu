@@ -337,10 +337,33 @@ __global__ void scatter_csr_kernel(const int64_t* __restrict__ dst, const double
     arena[dst[e]] += (real)val[e];
 }
 
+// The level-to-level copies sit between two sweeps that are programmatic
+// dependents of one another (kernels_apply.cu) and take part in the chain.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... KArgs, typename... Args>
+void launch_pdl(void (*kernel)(KArgs...), int grid, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  count_launch();
+  cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
 template <typename real>
 __global__ void gather_vec_kernel(const int64_t* __restrict__ idx, int64_t n,
                                   const real* __restrict__ src, int64_t lds, real* __restrict__ dst,
                                   int64_t ldd, int nrhs) {
+  pdl_begin();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * nrhs;
        e += (int64_t)gridDim.x * blockDim.x) {
     int64_t p = e % n;
@@ -353,6 +376,7 @@ template <typename real>
 __global__ void scatter_vec_kernel(const int64_t* __restrict__ idx, int64_t n,
                                    const real* __restrict__ src, int64_t lds,
                                    real* __restrict__ dst, int64_t ldd, int nrhs) {
+  pdl_begin();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * nrhs;
        e += (int64_t)gridDim.x * blockDim.x) {
     int64_t p = e % n;
@@ -551,16 +575,16 @@ template <typename real>
 void Launch<real>::gather_vec(const int64_t* idx, int64_t n, const real* src, int64_t lds,
                               real* dst, int64_t ldd, int nrhs, cudaStream_t st) {
   if (n <= 0) return;
-  count_launch();
-  gather_vec_kernel<real><<<grid_for(n * nrhs, 256), 256, 0, st>>>(idx, n, src, lds, dst, ldd, nrhs);
+  launch_pdl(gather_vec_kernel<real>, grid_for(n * nrhs, 256), st, idx, n, src, lds, dst, ldd,
+             nrhs);
 }
 
 template <typename real>
 void Launch<real>::scatter_vec(const int64_t* idx, int64_t n, const real* src, int64_t lds,
                                real* dst, int64_t ldd, int nrhs, cudaStream_t st) {
   if (n <= 0) return;
-  count_launch();
-  scatter_vec_kernel<real><<<grid_for(n * nrhs, 256), 256, 0, st>>>(idx, n, src, lds, dst, ldd, nrhs);
+  launch_pdl(scatter_vec_kernel<real>, grid_for(n * nrhs, 256), st, idx, n, src, lds, dst, ldd,
+             nrhs);
 }
 
 template <typename real>
