@@ -218,10 +218,20 @@ struct Launch {
   static size_t qr_cluster_smem(int maxm, int maxc, int CL);
   static void count_nz(const PrepTask* tasks_dev, int ntask, int maxc, const real* arena,
                        double* wsd, const Seg* segs, int* cnt, cudaStream_t st);
-  static void qr_cluster(const PrepTask* tasks_dev, int ntask, int maxm, int maxc, int CL,
-                         const real* arena, real* ws, double* wsd, const Seg* segs, int* rank,
-                         int* piv, const int* fpiv, const int* cnt, double eps, int max_rank,
-                         cudaStream_t st);
+  // (tasks order[0..ntask) of the list, cnt by task; likewise below)
+  static void qr_cluster(const PrepTask* tasks_dev, const int* order, int ntask, int maxm,
+                         int maxc, int CL, const real* arena, real* ws, double* wsd,
+                         const Seg* segs, int* rank, int* piv, const int* fpiv, const int* cnt,
+                         double eps, int max_rank, cudaStream_t st);
+  // the same with the columns in registers: the form for a task of m unknowns
+  // and c columns (-1 = none) and its cluster size, and the launch of tasks
+  // that share both; beside: may run beside the launch before it, which is one
+  // of the same class
+  static int qr_reg_form(int m, int c, int* CL);
+  static void qr_reg(int form, int CL, int maxc, bool beside, const PrepTask* tasks_dev,
+                     const int* order, int ntask, const real* arena, real* ws, double* wsd,
+                     const Seg* segs, int* rank, int* piv, const int* fpiv, const int* cnt,
+                     double eps, int max_rank, cudaStream_t st);
   static void sketch(const SketchTask* tasks_dev, int ntask, int maxm, int maxl,
                      const real* arena, real* ws, const Seg* segs,
                      cudaStream_t st);

@@ -11,6 +11,7 @@
 #include <condition_variable>
 #include <functional>
 #include <type_traits>
+#include <array>
 #include <atomic>
 #include <chrono>
 #include <thread>
@@ -21,6 +22,7 @@
 #include <mutex>
 #include <numeric>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "common.h"
@@ -1166,28 +1168,71 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
         HS_CUDA(cudaStreamSynchronize(h->st));
       }
       for (size_t i = 0; i < qrt.size(); i++) nzcols[qrt[i].s] = cnt[i];
-      const int nzmax = std::max(1, *std::max_element(cnt.begin(), cnt.end()));
-      int CL = Launch<real>::qr_cluster_size(qm, nzmax);
+      // The float32 SPD path keeps columns in registers (form, CTAs per
+      // cluster).  A class that fits the chip at once takes the form of its
+      // largest task; in a larger one every task takes the form its own size
+      // allows (96^3, level 1: 36.0 -> 22.7 ms; the launches run side by side,
+      // but each costs its start: grouping the one-wave classes of level 3 as
+      // well took 34.0 ms against 29.7).  What fits no form shares one launch
+      // that keeps the columns in shared memory.
+      int one_CL = 0;
+      const int nz_all = std::max(1, *std::max_element(cnt.begin(), cnt.end()));
+      const int one = sym ? Launch<real>::qr_reg_form(qm, nz_all, &one_CL) : -1;
+      const bool whole = one >= 0 && (int64_t)qrt.size() * one_CL <= kNumSMs;
+      std::vector<std::array<int, 3>> at;  // form (-1: shared memory), CTAs, task
+      int sm_m = 0, sm_nz = 0, sm_n = 0;
+      for (size_t i = 0; i < qrt.size(); i++) {
+        int CL = 0;
+        const int form =
+            whole ? one
+                  : sym ? Launch<real>::qr_reg_form(qrt[i].m, std::max(1, cnt[i]), &CL) : -1;
+        if (whole) CL = one_CL;
+        if (form < 0) {
+          sm_m = std::max(sm_m, qrt[i].m);
+          sm_nz = std::max(sm_nz, std::max(1, cnt[i]));
+          sm_n++;
+          CL = 0;
+        }
+        at.push_back({form, CL, (int)i});
+      }
+      int sm_CL = sm_n > 0 ? Launch<real>::qr_cluster_size(sm_m, sm_nz) : 1;
       // a class of few clusters spreads each block over more CTAs (up to the
       // portable cluster size 8, at least 64 columns each) to occupy the SMs
-      if (CL > 0)
-        while (CL < 8 && (int64_t)qrt.size() * CL * 2 <= 2 * kNumSMs && nzmax >= CL * 2 * 64)
-          CL *= 2;
-      if (CL > 0) {
+      if (sm_CL > 0)
+        while (sm_CL < 8 && (int64_t)sm_n * sm_CL * 2 <= 2 * kNumSMs && sm_nz >= sm_CL * 2 * 64)
+          sm_CL *= 2;
+      if (sm_CL > 0) {
+        // the widest clusters of CTAs first: they need the most SMs at once
+        std::sort(at.begin(), at.end(), [](const auto& x, const auto& y) {
+          return std::make_tuple(-x[1], x[0], x[2]) < std::make_tuple(-y[1], y[0], y[2]);
+        });
+        std::vector<int> order;
+        for (auto& e : at) order.push_back(e[2]);
         for (auto& pt : prep)
           if (pt.l == 0 && pt.ncolG > 0) pt.qr = 2;
         Blob b3;
-        size_t o3_prep = b3.add(prep);
+        size_t o3_prep = b3.add(prep), o3_ord = b3.add(order);
         h->blob3.ensure(std::max<size_t>(b3.h.size(), 16));
         h->pin3.ensure(std::max<size_t>(b3.h.size(), 16));
         std::memcpy(h->pin3.p, b3.h.data(), b3.h.size());
         HS_CUDA(cudaMemcpyAsync(h->blob3.p, h->pin3.p, b3.h.size(), cudaMemcpyHostToDevice,
                                 h->st));
         d_prep = reinterpret_cast<const PrepTask*>(h->blob3.as<char>() + o3_prep);
+        const int* d_ord = reinterpret_cast<const int*>(h->blob3.as<char>() + o3_ord);
         timed_lv(h, "qr_cluster", level, 1, [&] {
-          Launch<real>::qr_cluster(d_qrt, (int)qrt.size(), qm, nzmax, CL, arena, ws,
-                                   h->wsd.as<double>(), d_segs, rank, pivd, fpiv,
+          for (size_t i = 0, e = 0; i < at.size(); i = e) {
+            int nzm = 1;
+            for (e = i; e < at.size() && at[e][0] == at[i][0] && at[e][1] == at[i][1]; e++)
+              nzm = std::max(nzm, cnt[at[e][2]]);
+            if (at[i][0] >= 0)
+              Launch<real>::qr_reg(at[i][0], at[i][1], nzm, i > 0, d_qrt, d_ord + i, (int)(e - i),
+                                   arena, ws, h->wsd.as<double>(), d_segs, rank, pivd, fpiv,
                                    h->cnt.as<int>(), eps, max_rank_arg, h->st);
+            else
+              Launch<real>::qr_cluster(d_qrt, d_ord + i, (int)(e - i), sm_m, sm_nz, sm_CL, arena,
+                                       ws, h->wsd.as<double>(), d_segs, rank, pivd, fpiv,
+                                       h->cnt.as<int>(), eps, max_rank_arg, h->st);
+          }
         });
         if (!rank_in_prep) copy_ranks();
       }

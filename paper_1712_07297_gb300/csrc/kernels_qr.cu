@@ -2,16 +2,16 @@
 // spread over a thread-block cluster.
 //
 // The fill block G (m x c, c often in the thousands) is split by columns over
-// the CL CTAs of a cluster; each CTA keeps its nonzero columns in its own
-// shared memory for the whole factorization, so every step streams shared
-// memory instead of L2.  Per step the CTAs agree on the pivot through
-// distributed shared memory: the largest remaining column norm over the
-// cluster, then the lowest original column index among the columns within
-// 1e-10 of it (the tie rule of the single-CTA path); every CTA forms the
-// reflector from the pivot column in the owner's shared memory and updates
-// its columns.  Two cluster barriers per step; every CTA takes the same
-// branches (its decisions use the same exchanged values), so the barriers
-// always match.
+// the CL CTAs of a thread-block cluster.  qr_reg_kernel keeps the columns in
+// registers for the whole factorization (clusters of up to 256 unknowns, fill
+// blocks that 8 CTAs hold); qr_cluster_kernel keeps them in shared memory
+// (larger ones).  Per step the CTAs agree on the pivot through distributed
+// shared memory: the largest remaining column norm over the cluster, then the
+// lowest original column index among the columns within the tie tolerance of
+// it (the tie rule of the single-CTA path); the reflector is formed from the
+// pivot column and every CTA updates its columns.  Two cluster barriers per
+// step; every CTA takes the same branches (its decisions use the same
+// exchanged values), so the barriers always match.
 //
 // A count pass first flags and counts the nonzero gathered columns, so that
 // each CTA holds an equal share of the nonzero ones and the cluster size and
@@ -32,11 +32,6 @@ namespace hs {
 
 namespace {
 
-// near-ties of the pivot search, relative: 1e-10 in float64; in float32 the
-// squared norms carry ~1e-7 relative rounding, so ties of exact arithmetic
-// are recognised within 1e-5
-template <typename real>
-__device__ __forceinline__ double tie_rtol() { return sizeof(real) == 8 ? 1e-10 : 1e-5; }
 constexpr size_t kQrSmemCap = 200 * 1024;  // dynamic shared memory per CTA, at most
 constexpr int kQrThreads = 256;  // threads per CTA of the cluster QR (more only add barrier cost)
 constexpr int kMaxGrid = 1 << 20;
@@ -44,29 +39,87 @@ constexpr int kMaxGrid = 1 << 20;
 // Dynamic shared memory of one CTA: every array starts on a 16-byte boundary
 // (the same computation sizes the launch and carves the buffer).
 struct QrSmem {
-  size_t G, nrm, oidx, tpos, vloc, total;
+  size_t G, nrm, oidx, vloc, total;
   __host__ __device__ static size_t al(size_t b) { return (b + 15) / 16 * 16; }
   __host__ __device__ QrSmem(int ldsm, int cc, int sz) {
     G = 0;
     nrm = G + al((size_t)ldsm * cc * sz);
     oidx = nrm + al((size_t)cc * sizeof(double));
-    tpos = oidx + al((size_t)cc * sizeof(int));
-    vloc = tpos + al((size_t)kQrThreads * sizeof(int));
+    vloc = oidx + al((size_t)cc * sizeof(int));
     total = vloc + al((size_t)ldsm * sz);
   }
 };
 
+// Squared norms as keys: maxima of non-negative floating point numbers are
+// integer maxima of their bit patterns, one instruction per warp, and float32
+// stays off the float64 pipe (two lanes per clock on this chip).
+template <typename real>
+struct NormKey;
+template <>
+struct NormKey<float> {  // non-negative floats order as their bit patterns
+  using type = unsigned;
+  static __device__ __forceinline__ type of(float v) { return __float_as_uint(v); }
+  static __device__ __forceinline__ float value(type k) { return __uint_as_float(k); }
+  static __device__ __forceinline__ type warp_max(type k) {
+    return __reduce_max_sync(0xffffffffu, k);
+  }
+  // near-ties of the pivot search: squared norms carry ~1e-7 relative
+  // rounding, so ties of exact arithmetic are recognised within 1e-5
+  static __device__ __forceinline__ float band(float M) { return M * (1.0f - 1e-5f); }
+  // the largest float x with x <= v
+  static __device__ __forceinline__ float floor_of(double v) { return __double2float_rd(v); }
+};
+template <>
+struct NormKey<double> {
+  using type = unsigned long long;
+  static __device__ __forceinline__ type of(double v) { return __double_as_longlong(v); }
+  static __device__ __forceinline__ double value(type k) { return __longlong_as_double(k); }
+  static __device__ __forceinline__ type warp_max(type k) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+    const unsigned lo =
+        __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+    return ((type)hi << 32) | lo;
+  }
+  static __device__ __forceinline__ double band(double M) { return (1.0 - 1e-10) * M; }
+  static __device__ __forceinline__ double floor_of(double v) { return v; }
+};
+
+// Head x0 - beta (beta = -sign(x0) r) and tau = 1 / (r (r + |x0|)) of the
+// reflector of a column of squared norm r2.
+__device__ __forceinline__ void reflector(double r2, double x0, double* head, double* tau) {
+  const double r = sqrt(r2);
+  *head = x0 >= 0.0 ? x0 + r : x0 - r;
+  *tau = r > 0.0 ? 1.0 / (r * (r + fabs(x0))) : 0.0;
+}
+
+// The same with about 44 correct bits before the final rounding, in pairs of
+// floats (Dekker 1971: residuals of a square root, a sum and a product are
+// exact or nearly so with fma).
+__device__ __forceinline__ void reflector(float r2, float x0, float* head, float* tau) {
+  const float r = sqrtf(r2);
+  if (!(r > 0.f)) {
+    *head = x0;
+    *tau = 0.f;
+    return;
+  }
+  const float rl = fmaf(-r, r, r2) / (2.f * r);  // sqrt(r2) = r + rl
+  const float a = fabsf(x0);
+  const float h = r + a, t = h - r;                      // r + |x0| = h + hl
+  const float hl = ((r - (h - t)) + (a - t)) + rl;
+  const float q = r * h;                                 // r (r + |x0|) = q + ql
+  const float ql = fmaf(r, h, -q) + fmaf(r, hl, rl * h);
+  const float t0 = 1.f / q;
+  *tau = fmaf(t0, fmaf(-q, t0, 1.f) - ql * t0, t0);
+  *head = copysignf(h + hl, x0 >= 0.f ? 1.f : -1.f);
+}
+
+template <typename real>
 struct Exchange {
-  double val;      // largest local squared norm
-  double candnrm;  // squared norm of the local candidate
+  real val;        // largest local squared norm
+  real candnrm;    // squared norm of the local candidate
   int cand;        // lowest original index among the local candidates
   int loc;         // local column of the candidate
 };
-
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 
 __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -76,21 +129,10 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
   return v;
 }
 
-__device__ double block_max(double v, double* red) {
-  red[threadIdx.x] = v;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
-    __syncthreads();
-  }
-  double r = red[0];
-  __syncthreads();
-  return r;
-}
-
 template <typename real>
 __global__ void __launch_bounds__(kQrThreads)
-qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ arena,
+qr_cluster_kernel(const PrepTask* __restrict__ tasks, const int* __restrict__ order,
+                  const real* __restrict__ arena,
                   real* __restrict__ ws_all, double* __restrict__ wsd_all,
                   const Seg* __restrict__ segs, int* rank, int* __restrict__ piv,
                   const int* __restrict__ fpiv, const int* __restrict__ cnt, double eps,
@@ -98,16 +140,18 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
   cg::cluster_group cl = cg::this_cluster();
   const int CL = (int)cl.num_blocks();
   const int cr = (int)cl.block_rank();
-  const PrepTask tk = tasks[blockIdx.x / CL];
+  const int task = order[blockIdx.x / CL];
+  const PrepTask tk = tasks[task];
   const int m = tk.m, c = tk.ncolG;
-  __shared__ double red_d[kQrThreads];
-  __shared__ Exchange xch;
+  using Key = NormKey<real>;
+  __shared__ real red_n[kQrThreads / 32];
+  __shared__ int scan[kQrThreads / 32];
+  __shared__ Exchange<real> xch;
   extern __shared__ __align__(16) unsigned char dsm[];
   const QrSmem lay(ldsm, ccmax, (int)sizeof(real));
   real* Gs = reinterpret_cast<real*>(dsm + lay.G);  // ldsm x ccmax, column-major
-  double* nrm = reinterpret_cast<double*>(dsm + lay.nrm);
+  real* nrm = reinterpret_cast<real*>(dsm + lay.nrm);
   int* oidx = reinterpret_cast<int*>(dsm + lay.oidx);
-  int* tpos = reinterpret_cast<int*>(dsm + lay.tpos);
   real* vloc = reinterpret_cast<real*>(dsm + lay.vloc);  // the step's reflector
 
   // per-cluster outputs (same layout as the per-cluster kernel)
@@ -117,40 +161,41 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
   real* W_G = ws_all + tk.ws + 10 * (int64_t)m * m;
 
   // scale of the rounding-noise floor: max |A_ss|
-  double amx = 0;
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x)
-    amx = fmax(amx, fabs((double)arena[tk.a_ss + idx % m + (int64_t)(idx / m) * tk.ld]));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  real amx = 0;
+  for (int j = warp; j < m; j += nwarp)
+    for (int i = lane; i < m; i += 32) amx = fmax(amx, fabs(arena[tk.a_ss + i + (int64_t)j * tk.ld]));
+  amx = Key::value(Key::warp_max(Key::of(amx)));
+  if (lane == 0) red_n[warp] = amx;
+  __syncthreads();
+  for (int w = 0; w < nwarp; w++) amx = fmax(amx, red_n[w]);
   // forced ranks keep every direction up to the forced count (no floor)
-  const double floor = max_rank < 0 ? 0.0 : noise_rtol * block_max(amx, red_d);
+  const double floor = max_rank < 0 ? 0.0 : noise_rtol * (double)amx;
 
   // The count pass flagged the nonzero gathered columns (flags[q] != 0) and
   // counted them (nz); CTA cr keeps nonzero columns cr*cz .. (cr+1)*cz - 1
   // in gathered order, so every CTA holds at most cz columns.
-  const double* flags = nrm2_g + tk.ncolG;
-  const int nz = cnt[blockIdx.x / CL];
+  const int* flags = reinterpret_cast<const int*>(nrm2_g + tk.ncolG);
+  const int nz = cnt[task];
   const int cz = (nz + CL - 1) / CL;
   const int z0 = cr * cz, z1 = min(nz, z0 + cz);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   {
     const int per = (c + blockDim.x - 1) / blockDim.x;
     const int a0 = min(c, (int)threadIdx.x * per), a1 = min(c, a0 + per);
     int n = 0;
-    for (int q = a0; q < a1; q++) n += (flags[q] != 0.0);
-    tpos[threadIdx.x] = n;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int acc = 0;
-      for (int t = 0; t < (int)blockDim.x; t++) {
-        const int v = tpos[t];
-        tpos[t] = acc;
-        acc += v;
-      }
+    for (int q = a0; q < a1; q++) n += flags[q];
+    int inc = n;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
     }
+    if (lane == 31) scan[warp] = inc;
     __syncthreads();
-    int zq = tpos[threadIdx.x];
+    int zq = inc - n;
+    for (int w = 0; w < warp; w++) zq += scan[w];
     // the gathered column of each of this CTA's slots
     for (int q = a0; q < a1; q++) {
-      if (flags[q] == 0.0) continue;
+      if (flags[q] == 0) continue;
       if (zq >= z0 && zq < z1) oidx[zq - z0] = q;
       zq++;
     }
@@ -172,7 +217,7 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
       const real x = Gs[i + (int64_t)t * ldsm];
       s += x * x;
     }
-    nrm[t] = (double)s;
+    nrm[t] = s;
   }
   __syncthreads();
 
@@ -181,39 +226,40 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
   const int kmax = max_rank > 0 ? min(m, max_rank) : (max_rank < 0 ? min(m, rank[tk.s]) : m);
   if (max_rank < 0) eps = 0.0;
   const int steps = min(m, c);
-  double r11 = 0;
+  real stop = 0;  // a squared norm at or below this ends the factorization
   int k = 0;
   __shared__ unsigned long long red_u[kQrThreads / 32];
-  __shared__ double s_M, s_r;
+  __shared__ real s_M, s_r2;
   __shared__ int s_owner;
   for (int j = 0; j < steps; j++) {
     // 1. largest remaining norm over the cluster
-    double lmx = 0;
+    real lmx = 0;
     for (int t = threadIdx.x; t < nloc; t += blockDim.x) lmx = fmax(lmx, nrm[t]);
-    lmx = warp_max(lmx);
-    if (lane == 0) red_d[warp] = lmx;
+    lmx = Key::value(Key::warp_max(Key::of(lmx)));
+    if (lane == 0) red_n[warp] = lmx;
     __syncthreads();
     if (threadIdx.x == 0) {
-      double v = red_d[0];
-      for (int w = 1; w < nwarp; w++) v = fmax(v, red_d[w]);
+      real v = red_n[0];
+      for (int w = 1; w < nwarp; w++) v = fmax(v, red_n[w]);
       xch.val = v;
     }
     cl.sync();
     if (warp == 0) {
-      double v = (lane < CL) ? cl.map_shared_rank(&xch, lane)->val : 0.0;
-      v = warp_max(v);
-      if (lane == 0) s_M = v;
+      const real v = (lane < CL) ? cl.map_shared_rank(&xch, lane)->val : real(0);
+      const real x = Key::value(Key::warp_max(Key::of(v)));
+      if (lane == 0) s_M = x;
     }
     __syncthreads();
-    const double M = s_M;
-    if (M <= 0.0) break;
+    const real M = s_M;
+    if (!(M > real(0))) break;
+    const real band = Key::band(M);
     // 2. lowest original index among the near-maximal columns: one key
     //    (original index, local slot) per candidate, the smallest wins; a
     //    given pivot order (fpiv) makes its column the only candidate
     unsigned long long key = ~0ull;
     const int fq = fpiv ? fpiv[tk.pv + j] : -1;
     for (int t = threadIdx.x; t < nloc; t += blockDim.x)
-      if (fpiv ? (z0 + t == fq && nrm[t] >= 0.0) : (nrm[t] >= (1.0 - tie_rtol<real>()) * M)) {
+      if (fpiv ? (z0 + t == fq && nrm[t] >= real(0)) : (nrm[t] >= band)) {
         const unsigned long long kk = ((unsigned long long)oidx[t] << 32) | (unsigned)t;
         key = kk < key ? kk : key;
       }
@@ -226,7 +272,7 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
       const bool any = v != ~0ull;
       xch.cand = any ? (int)(v >> 32) : INT_MAX;
       xch.loc = any ? (int)(v & 0xffffffffu) : -1;
-      xch.candnrm = any ? nrm[(int)(v & 0xffffffffu)] : -1.0;
+      xch.candnrm = any ? nrm[(int)(v & 0xffffffffu)] : real(-1);
     }
     cl.sync();
     if (warp == 0) {
@@ -236,33 +282,38 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
       v = warp_min_u64(v);
       if (lane == 0) {
         s_owner = (int)(v & 0xff);
-        s_r = sqrt(cl.map_shared_rank(&xch, (int)(v & 0xff))->candnrm);
+        s_r2 = cl.map_shared_rank(&xch, (int)(v & 0xff))->candnrm;
       }
     }
     __syncthreads();
     const int owner = s_owner;
-    const double r = s_r;
-    if (!(r >= 0.0)) break;  // a given pivot that names no remaining column
-    if (j == 0) r11 = r;
-    if (r <= floor || (eps > 0.0 && r <= eps * r11) || j >= kmax) break;
+    const real r2 = s_r2;
+    if (!(r2 >= real(0))) break;  // a given pivot that names no remaining column
+    if (j == 0) {
+      // |r_jj| <= floor or |r_jj| <= eps |r_11|, on the squares
+      double s2 = floor * floor;
+      if (eps > 0.0) s2 = fmax(s2, eps * eps * (double)r2);
+      stop = Key::floor_of(s2);
+    }
+    if (r2 <= stop || j >= kmax) break;
     // 3. every CTA forms the reflector v = x - beta e1, beta = -sign(x0) ||x||
     //    from the pivot column in the owner's shared memory (read through
     //    distributed shared memory; that column is never written again, so
     //    no further cluster barrier is needed); the owner also stores it
     const int oloc = cl.map_shared_rank(&xch, owner)->loc;
     const real* ocol = cl.map_shared_rank(Gs, owner) + (int64_t)oloc * ldsm;
-    const double x0 = (double)ocol[j];
-    const double beta = (x0 >= 0.0) ? -r : r;
-    const real tj = (real)((r > 0.0) ? 1.0 / (r * (r + fabs(x0))) : 0.0);
+    const real x0 = ocol[j];
+    real head, tj;
+    reflector(r2, x0, &head, &tj);
     for (int i = j + threadIdx.x; i < m; i += blockDim.x) {
-      const real v = (i == j) ? (real)(x0 - beta) : ocol[i];
+      const real v = (i == j) ? head : ocol[i];
       vloc[i] = v;
       if (cr == owner) W_G[i + (int64_t)j * m] = v;
     }
     if (cr == owner && threadIdx.x == 0) {
       tau_g[j] = tj;
-      rsign_g[j] = beta < 0.0 ? real(-1) : real(1);
-      nrm[oloc] = -1.0;  // used: out of every later step
+      rsign_g[j] = x0 >= real(0) ? real(-1) : real(1);
+      nrm[oloc] = real(-1);  // used: out of every later step
       // the pivot as an index among the nonzero gathered columns: slot t of
       // CTA cr holds nonzero column z0 + t
       piv[tk.pv + j] = z0 + oloc;
@@ -271,7 +322,7 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
     // 4. every CTA applies the reflector to its remaining columns and
     //    recomputes their squared norms over rows j+1..m
     for (int t = threadIdx.x; t < nloc; t += blockDim.x) {
-      if (nrm[t] < 0.0) continue;
+      if (nrm[t] < real(0)) continue;
       real* col = Gs + (int64_t)t * ldsm;
       // four independent partial sums (combined in a fixed order) keep four
       // products in flight instead of one dependent chain
@@ -305,7 +356,7 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
         col[i] = a;
         s0 += a * a;
       }
-      nrm[t] = (double)((s0 + s1) + (s2 + s3));
+      nrm[t] = (s0 + s1) + (s2 + s3);
     }
     __syncthreads();
     k = j + 1;
@@ -313,6 +364,282 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ a
   if (cr == 0 && threadIdx.x == 0) rank[tk.s] = k;
   // no CTA leaves while another may still read its shared memory
   cl.sync();
+}
+
+// ---------------------------------------------------------------------------
+// Register-resident pivoted QR
+// ---------------------------------------------------------------------------
+// TPC threads share a column, thread h of them rows h, h + TPC, .. (RPT of
+// them, zero beyond m), so a step reads only the reflector from shared memory
+// (16-byte broadcasts) where the shared-memory form reads each element twice,
+// writes it once and reads two scalars of the reflector beside it.  What else a
+// step pays for is latency, so: columns lie on the warps in gathered order,
+// and the winner -- the lowest index within the tie band of the largest norm
+// -- is in the first warp whose own maximum reaches the band, found without a
+// second reduction (two CTA barriers per step; with several CTAs one and two
+// cluster barriers); and float32 stays off the float64 pipe (two lanes per
+// clock on this chip): norms compare as integers, thresholds are rounded to
+// float32 once, the reflector's scalars are formed in float32 pairs.  (The
+// float64 path is bound by that pipe, 56,000 products per step and SM at 128 x
+// 280, and keeps the shared-memory form, whose rows end exactly at m; so does
+// the float32 general path.)  Per step: search 1.0 us, publish 1.2-1.6, apply
+// 1.1-1.3 (two cluster barriers among them; the shared-memory form took 6 to
+// 8).  All fill blocks of a factorization, shared memory -> registers: 64^3
+// 47.5 -> 20 ms, 96^3 184 -> 99 ms.
+// CTAs of a thread-block cluster: 16 (beyond the portable 8) hold the coarse
+// levels' widest fill blocks
+constexpr int kRegMaxCl = 16;
+
+template <typename real, int RPT, int TPC, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+qr_reg_kernel(const PrepTask* __restrict__ tasks, const int* __restrict__ order,
+              const real* __restrict__ arena,
+              real* __restrict__ ws_all, double* __restrict__ wsd_all,
+              const Seg* __restrict__ segs, int* rank, int* __restrict__ piv,
+              const int* __restrict__ fpiv, const int* __restrict__ cnt, double eps,
+              double noise_rtol, int max_rank) {
+  using Key = NormKey<real>;
+  using key_t = typename Key::type;
+  constexpr int kBlk = 8, kBlocks = RPT / kBlk;
+  constexpr int kPad = 16 / (int)sizeof(real);  // threads of a column on other banks
+  constexpr int kLdv = RPT + kPad;
+  // the launches of a class run beside one another: each lets the next one
+  // start at once and ends only after the one before it has
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), cr = (int)cl.block_rank();
+  const int task = order[blockIdx.x / CL];
+  const PrepTask tk = tasks[task];
+  const int m = tk.m, c = tk.ncolG;
+  // the step's reflector, by thread of a column, then its squared norm, its
+  // tau and the pivot's index
+  constexpr int kInfo = TPC * kLdv, kVs = kInfo + kPad;
+  __shared__ __align__(16) real vs[2][kVs];
+  __shared__ key_t wmax[2][32];                     // largest norm of every warp
+  __shared__ key_t xmax[2][kRegMaxCl];              // and of every CTA
+  __shared__ int scan[33];
+  __shared__ int slot_col[NT / TPC];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int t = threadIdx.x / TPC, h = threadIdx.x % TPC;
+
+  double* nrm2_g = wsd_all + tk.wsd;
+  real* tau_g = reinterpret_cast<real*>(nrm2_g + 2 * (int64_t)tk.ncolG);
+  real* rsign_g = tau_g + 2 * m;
+  real* W_G = ws_all + tk.ws + 10 * (int64_t)m * m;
+
+  // this CTA's columns: nonzero columns cr * cz .. (cr + 1) * cz - 1 in
+  // gathered order, one per slot
+  const int* flags = reinterpret_cast<const int*>(nrm2_g + tk.ncolG);
+  const int nz = cnt[task];
+  const int cz = (nz + CL - 1) / CL;
+  const int z0 = min(nz, cr * cz), z1 = min(nz, z0 + cz), nloc = z1 - z0;
+  {
+    const int per = (c + blockDim.x - 1) / blockDim.x;
+    const int a0 = min(c, (int)threadIdx.x * per), a1 = min(c, a0 + per);
+    int n = 0;
+    for (int q = a0; q < a1; q++) n += flags[q];
+    int inc = n;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) scan[warp] = inc;
+    __syncthreads();
+    int before = inc - n;
+    for (int w = 0; w < warp; w++) before += scan[w];
+    for (int q = a0; q < a1; q++) {
+      if (flags[q] == 0) continue;
+      if (before >= z0 && before < z1) slot_col[before - z0] = q;
+      before++;
+    }
+    __syncthreads();
+  }
+  real col[RPT];
+#pragma unroll
+  for (int r = 0; r < RPT; r++) col[r] = 0;
+  if (t < nloc) {
+    int64_t p;
+    int st;
+    seg_col(segs + tk.gcol, tk.ngcol, slot_col[t], &p, &st);
+#pragma unroll
+    for (int r = 0; r < RPT; r++) {
+      const int i = r * TPC + h;
+      if (i < m) col[r] = arena[p + (int64_t)i * st];
+    }
+  }
+  // scale of the rounding-noise floor: max |A_ss|
+  real amx = 0;
+  for (int j = warp; j < m; j += 4 * nwarp)
+    for (int i = lane; i < m; i += 32) {
+      real x[4];
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        x[q] = j + q * nwarp < m ? arena[tk.a_ss + i + (int64_t)(j + q * nwarp) * tk.ld] : real(0);
+#pragma unroll
+      for (int q = 0; q < 4; q++) amx = fmax(amx, fabs(x[q]));
+    }
+  const auto column_sum = [](real s) {
+#pragma unroll
+    for (int o = 1; o < TPC; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  };
+  real nrm;
+  {
+    real s[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int r = 0; r < RPT; r++) s[r & 3] += col[r] * col[r];
+    nrm = column_sum((s[0] + s[1]) + (s[2] + s[3]));
+  }
+  {
+    const key_t a = Key::warp_max(Key::of(amx));
+    if (lane == 0) wmax[1][warp] = a;
+  }
+  __syncthreads();
+  amx = Key::value(Key::warp_max(lane < nwarp ? wmax[1][lane] : key_t(0)));
+  // forced ranks keep every direction up to the forced count (no floor)
+  const double floor = max_rank < 0 ? 0.0 : noise_rtol * (double)amx;
+  const int kmax = max_rank > 0 ? min(m, max_rank) : (max_rank < 0 ? min(m, rank[tk.s]) : m);
+  if (max_rank < 0) eps = 0.0;
+  const int steps = min(m, c);
+  const int nblk = (m + kBlk * TPC - 1) / (kBlk * TPC);  // row blocks that hold rows
+  real stop = 0;  // a squared norm at or below this ends the factorization
+  bool used = false;
+  int k = 0;
+  cl.sync();  // rank[s] is read, and every CTA runs before its memory is written
+  for (int j = 0; j < steps; j++) {
+    const int par = j & 1;
+    // 1. largest remaining norm, and which warp's columns hold the pivot
+    const key_t mine = used ? key_t(0) : Key::of(nrm);
+    const key_t wm = Key::warp_max(mine);
+    if (lane == 0) wmax[par][warp] = wm;
+    __syncthreads();
+    const key_t wl = lane < nwarp ? wmax[par][lane] : key_t(0);
+    key_t M = Key::warp_max(wl);
+    int owner = 0;
+    const int fq = fpiv ? fpiv[tk.pv + j] : -1;
+    if (CL > 1) {
+      if (warp == 0 && lane < CL) *cl.map_shared_rank(&xmax[par][cr], lane) = M;
+      cl.sync();
+      const key_t xl = lane < CL ? xmax[par][lane] : key_t(0);
+      M = Key::warp_max(xl);
+      owner = __ffs(__ballot_sync(0xffffffffu, lane < CL && Key::value(xl) >=
+                                                              Key::band(Key::value(M)))) - 1;
+    }
+    if (!(Key::value(M) > real(0))) break;
+    const real band = Key::band(Key::value(M));
+    int ww;
+    if (fpiv) {  // a given pivot order names its column
+      if (fq < 0 || fq >= nz) break;
+      owner = fq / cz;
+      ww = (fq - owner * cz) * TPC / 32;
+    } else {
+      ww = __ffs(__ballot_sync(0xffffffffu, lane < nwarp && Key::value(wl) >= band)) - 1;
+    }
+    // 2. the winner's warp publishes the reflector
+    if (cr == owner && warp == ww) {
+      const bool cand = fpiv ? (z0 + t == fq) : (!used && nrm >= band);
+      const int src = (__ffs(__ballot_sync(0xffffffffu, cand)) - 1) / TPC * TPC;
+      const bool win = lane / TPC * TPC == src;
+      if (win) {
+#pragma unroll
+        for (int r = 0; r < RPT; r++)
+          vs[par][h * kLdv + r] = r * TPC + h >= j ? col[r] : real(0);
+      }
+      __syncwarp();
+      const real x0 = vs[par][(j % TPC) * kLdv + j / TPC];
+      const real r2 = __shfl_sync(0xffffffffu, used ? real(-1) : nrm, src);
+      __syncwarp();
+      real head, tau;
+      reflector(r2, x0, &head, &tau);
+      if (lane == 0) {
+        vs[par][(j % TPC) * kLdv + j / TPC] = head;
+        vs[par][kInfo] = r2;
+        vs[par][kInfo + 1] = tau;
+      }
+      if (lane == src) vs[par][kInfo + 2] = __int_as_float(z0 + t);
+      __syncwarp();
+      if (CL > 1) {
+        // into the other CTAs' shared memory, 16 bytes at a time
+        constexpr int kUnits = kVs / kPad;
+        for (int e = lane; e < kUnits * CL; e += 32) {
+          const int q = e / kUnits, u = e % kUnits * kPad;
+          if (q != cr)
+            *reinterpret_cast<int4*>(cl.map_shared_rank(&vs[par][0], q) + u) =
+                *reinterpret_cast<const int4*>(&vs[par][u]);
+        }
+      }
+      used = used || win;
+    }
+    if (CL > 1) cl.sync();
+    else __syncthreads();
+    const real r2 = vs[par][kInfo];
+    if (!(r2 >= real(0))) break;  // a given pivot that is used already
+    if (j == 0) {
+      // |r_jj| <= floor or |r_jj| <= eps |r_11|, on the squares
+      double s2 = floor * floor;
+      if (eps > 0.0) s2 = fmax(s2, eps * eps * (double)r2);
+      stop = Key::floor_of(s2);
+    }
+    if (r2 <= stop || j >= kmax) break;
+    // the reflector leaves for the per-cluster kernel behind the barrier, from
+    // the CTAs in turn: a barrier waits for the stores before it
+    if (cr == j % CL) {
+      for (int i = j + threadIdx.x; i < m; i += blockDim.x)
+        W_G[i + (int64_t)j * m] = vs[par][(i % TPC) * kLdv + i / TPC];
+      if (threadIdx.x == 0) {
+        tau_g[j] = vs[par][kInfo + 1];
+        rsign_g[j] = vs[par][(j % TPC) * kLdv + j / TPC] >= real(0) ? real(-1) : real(1);
+        piv[tk.pv + j] = __float_as_int(vs[par][kInfo + 2]);
+      }
+    }
+    // 3. apply it to the remaining columns; squared norms of rows j+1..m (row
+    //    j of a column is not needed again and set to zero)
+    const real tau = vs[par][kInfo + 1];
+    const real* v = &vs[par][h * kLdv];
+    const int jb = j / (kBlk * TPC);
+    real w[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int b = 0; b < kBlocks; b++) {
+      if (b < jb || b >= nblk) continue;
+      real x[kBlk];
+#pragma unroll
+      for (int q = 0; q < kBlk; q += kPad)
+        *reinterpret_cast<int4*>(x + q) = *reinterpret_cast<const int4*>(v + b * kBlk + q);
+#pragma unroll
+      for (int q = 0; q < kBlk; q++) w[q & 3] += x[q] * col[b * kBlk + q];
+    }
+    const real wt = column_sum((w[0] + w[1]) + (w[2] + w[3])) * tau;
+    real s[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int b = 0; b < kBlocks; b++) {
+      if (b < jb || b >= nblk) continue;
+      real x[kBlk];
+#pragma unroll
+      for (int q = 0; q < kBlk; q += kPad)
+        *reinterpret_cast<int4*>(x + q) = *reinterpret_cast<const int4*>(v + b * kBlk + q);
+      if (b == jb) {
+#pragma unroll
+        for (int q = 0; q < kBlk; q++) {
+          const real a = (b * kBlk + q) * TPC + h > j ? col[b * kBlk + q] - wt * x[q] : real(0);
+          col[b * kBlk + q] = a;
+          s[q & 3] += a * a;
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < kBlk; q++) {
+          const real a = col[b * kBlk + q] - wt * x[q];
+          col[b * kBlk + q] = a;
+          s[q & 3] += a * a;
+        }
+      }
+    }
+    nrm = column_sum((s[0] + s[1]) + (s[2] + s[3]));
+    k = j + 1;
+  }
+  if (cr == 0 && threadIdx.x == 0) rank[tk.s] = k;
+  // no CTA leaves while another may still write its shared memory
+  cl.sync();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Count pass: flag the nonzero gathered columns of every task (flags in the
@@ -324,7 +651,7 @@ __global__ void __launch_bounds__(256)
 count_nz_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ arena,
                 double* __restrict__ wsd_all, const Seg* __restrict__ segs, int* cnt) {
   const PrepTask tk = tasks[blockIdx.x];
-  double* flags = wsd_all + tk.wsd + tk.ncolG;
+  int* flags = reinterpret_cast<int*>(wsd_all + tk.wsd + tk.ncolG);
   __shared__ int red[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   int n = 0;
@@ -341,7 +668,7 @@ count_nz_kernel(const PrepTask* __restrict__ tasks, const real* __restrict__ are
 #pragma unroll
       for (int r = 0; r < 8; r++) nz |= (x[r] != real(0));
     }
-    flags[q] = nz ? 1.0 : 0.0;
+    flags[q] = nz ? 1 : 0;
     n += nz;
   }
   for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
@@ -385,8 +712,8 @@ size_t Launch<real>::qr_cluster_smem(int maxm, int maxc, int CL) {
 }
 
 template <typename real>
-void Launch<real>::qr_cluster(const PrepTask* tasks_dev, int ntask, int maxm, int maxc, int CL,
-                              const real* arena, real* ws, double* wsd, const Seg* segs,
+void Launch<real>::qr_cluster(const PrepTask* tasks_dev, const int* order, int ntask, int maxm,
+                              int maxc, int CL, const real* arena, real* ws, double* wsd, const Seg* segs,
                               int* rank, int* piv, const int* fpiv, const int* cnt, double eps,
                               int max_rank, cudaStream_t st) {
   if (ntask <= 0) return;
@@ -419,8 +746,93 @@ void Launch<real>::qr_cluster(const PrepTask* tasks_dev, int ntask, int maxm, in
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     count_launch();
-    cudaLaunchKernelEx(&cfg, qr_cluster_kernel<real>, tasks_dev + t0, arena, ws, wsd, segs, rank,
-                       piv, fpiv, cnt + t0, eps, noise_rtol, max_rank, (maxm + 1) | 1, cc);
+    cudaLaunchKernelEx(&cfg, qr_cluster_kernel<real>, tasks_dev, order + t0, arena, ws, wsd, segs, rank,
+                       piv, fpiv, cnt, eps, noise_rtol, max_rank, (maxm + 1) | 1, cc);
+  }
+}
+
+namespace {
+// The forms of the register kernel (float32): rows per thread, threads per
+// column, most threads and CTAs per SM the registers are cut for.  The first
+// form with room for the class is taken: fewer rows per thread make a shorter
+// step, more threads per column leave fewer columns per CTA.
+struct QrForm {
+  int maxm, tpc, threads;
+  int cols() const { return threads / tpc; }
+};
+constexpr QrForm kQrForms[] = {{32, 4, 1024},  {32, 2, 1024}, {64, 4, 1024}, {64, 2, 1024},
+                               {128, 4, 576}, {128, 2, 576}, {256, 4, 512}};
+
+// The form for clusters of up to m unknowns and c columns, and its cluster
+// size (a portable one of any form before a larger one); -1 when none has
+// room.
+int reg_form(int m, int c, int* CL) {
+  for (int most = 8; most <= kRegMaxCl; most *= 2)
+    for (int i = 0; i < (int)(sizeof(kQrForms) / sizeof(kQrForms[0])); i++)
+      for (*CL = 1; m <= kQrForms[i].maxm && *CL <= most; *CL *= 2)
+        if ((c + *CL - 1) / *CL <= kQrForms[i].cols()) return i;
+  return -1;
+}
+
+template <typename real, int RPT, int TPC, int NT, int MINB>
+void launch_qr_reg(int CL, int cols, bool beside, const PrepTask* tasks, const int* order,
+                   int ntask, const real* arena, real* ws, double* wsd, const Seg* segs, int* rank,
+                   int* piv, const int* fpiv, const int* cnt, double eps, double noise,
+                   int max_rank, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  static const bool limit_set = [] {
+    cudaFuncSetAttribute(qr_reg_kernel<real, RPT, TPC, NT, MINB>,
+                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return true;
+  }();
+  (void)limit_set;
+  cfg.blockDim = dim3(std::max(64, (cols * TPC + 31) / 32 * 32));
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  for (int t0 = 0; t0 < ntask; t0 += 4096) {
+    attr[1].val.programmaticStreamSerializationAllowed = beside || t0 > 0;
+    cfg.gridDim = dim3(std::min(4096, ntask - t0) * CL);
+    count_launch();
+    cudaLaunchKernelEx(&cfg, qr_reg_kernel<real, RPT, TPC, NT, MINB>, tasks, order + t0, arena, ws,
+                       wsd, segs, rank, piv, fpiv, cnt, eps, noise, max_rank);
+  }
+}
+}  // namespace
+
+template <typename real>
+int Launch<real>::qr_reg_form(int m, int c, int* CL) {
+  return sizeof(real) == 4 ? reg_form(m, c, CL) : -1;
+}
+
+template <typename real>
+void Launch<real>::qr_reg(int form, int CL, int maxc, bool beside, const PrepTask* tasks,
+                          const int* order, int ntask, const real* arena, real* ws, double* wsd,
+                          const Seg* segs, int* rank, int* piv, const int* fpiv, const int* cnt,
+                          double eps, int max_rank, cudaStream_t st) {
+  if (ntask <= 0) return;
+  const int cols = std::max(1, (maxc + CL - 1) / CL);
+  const auto go = [&](auto launch) {
+    launch(CL, cols, beside, tasks, order, ntask, arena, ws, wsd, segs, rank, piv, fpiv, cnt, eps,
+           1e-6, max_rank, st);
+  };
+  if constexpr (sizeof(real) == 4) {
+    switch (form) {
+      case 0: go(launch_qr_reg<real, 8, 4, 1024, 1>); break;
+      case 1: go(launch_qr_reg<real, 16, 2, 1024, 1>); break;
+      case 2: go(launch_qr_reg<real, 16, 4, 1024, 1>); break;
+      case 3: go(launch_qr_reg<real, 32, 2, 1024, 1>); break;
+      case 4: go(launch_qr_reg<real, 32, 4, 576, 2>); break;
+      case 5: go(launch_qr_reg<real, 64, 2, 576, 1>); break;
+      case 6: go(launch_qr_reg<real, 64, 4, 512, 1>); break;
+      default: break;
+    }
   }
 }
 
