@@ -96,6 +96,37 @@ __host__ __device__ inline void seg_col(const Seg* sg, int nseg, int j, int64_t*
   }
 }
 
+#ifdef __CUDACC__
+// Head x0 - beta (beta = -sign(x0) r) and tau = 1 / (r (r + |x0|)) of the
+// reflector of a column of squared norm r2.
+__device__ __forceinline__ void householder_scalars(double r2, double x0, double* head, double* tau) {
+  const double r = sqrt(r2);
+  *head = x0 >= 0.0 ? x0 + r : x0 - r;
+  *tau = r > 0.0 ? 1.0 / (r * (r + fabs(x0))) : 0.0;
+}
+
+// The same with about 44 correct bits before the final rounding, in pairs of
+// floats (Dekker 1971: residuals of a square root, a sum and a product are
+// exact or nearly so with fma).
+__device__ __forceinline__ void householder_scalars(float r2, float x0, float* head, float* tau) {
+  const float r = sqrtf(r2);
+  if (!(r > 0.f)) {
+    *head = x0;
+    *tau = 0.f;
+    return;
+  }
+  const float rl = fmaf(-r, r, r2) / (2.f * r);  // sqrt(r2) = r + rl
+  const float a = fabsf(x0);
+  const float h = r + a, t = h - r;                      // r + |x0| = h + hl
+  const float hl = ((r - (h - t)) + (a - t)) + rl;
+  const float q = r * h;                                 // r (r + |x0|) = q + ql
+  const float ql = fmaf(r, h, -q) + fmaf(r, hl, rl * h);
+  const float t0 = 1.f / q;
+  *tau = fmaf(t0, fmaf(-q, t0, 1.f) - ql * t0, t0);
+  *head = copysignf(h + hl, x0 >= 0.f ? 1.f : -1.f);
+}
+#endif
+
 // Per-cluster task of the dense "prep" phase.
 struct PrepTask {
   int s;            // level-local cluster id
@@ -212,6 +243,11 @@ struct Launch {
                    int* rank, int* piv, const int* fpiv, double eps, int sym, int max_rank,
                    int maxm,
                    DevError* err, int level, long long* dbg, cudaStream_t st);
+  // the same for an SPD factorization whose pivoted QRs have run (or have no
+  // columns); false, nothing launched, for clusters above its limit
+  static bool prep_spd(const PrepTask* tasks_dev, int ntask, real* arena, real* fac, real* ws,
+                       double* wsd, int* rank, int maxm, DevError* err, int level,
+                       cudaStream_t st);
   // thread-block-cluster pivoted QR: cluster size for the largest task (0 =
   // does not fit), its dynamic shared memory, and the launch
   static int qr_cluster_size(int maxm, int maxc);

@@ -1248,7 +1248,13 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
       HS_CUDA(cudaMemsetAsync(h->dbg.p, 0, sizeof(long long) * 8 * (size_t)nt, h->st));
       dbg = h->dbg.as<long long>();
     }
+    // with every pivoted QR done, the SPD path has a kernel of its own
+    bool spd = sym && h->opts.cluster_qr && sk.empty();
+    for (auto& pt : prep) spd = spd && (pt.qr == 2 || pt.ncolG == 0);
     timed_lv(h, "prep", level, 1, [&] {
+      if (spd && Launch<real>::prep_spd(d_prep, nt, arena, fac, ws, h->wsd.as<double>(), rank,
+                                        maxm, h->d_err.as<DevError>(), level, h->st))
+        return;
       Launch<real>::prep(d_prep, nt, arena, fac, ws,
                          h->wsd.as<double>(), d_segs, rank, pivd, fpiv, eps, sym ? 1 : 0,
                          max_rank_arg, maxm, h->d_err.as<DevError>(), level, dbg, h->st);

@@ -84,35 +84,6 @@ struct NormKey<double> {
   static __device__ __forceinline__ double floor_of(double v) { return v; }
 };
 
-// Head x0 - beta (beta = -sign(x0) r) and tau = 1 / (r (r + |x0|)) of the
-// reflector of a column of squared norm r2.
-__device__ __forceinline__ void reflector(double r2, double x0, double* head, double* tau) {
-  const double r = sqrt(r2);
-  *head = x0 >= 0.0 ? x0 + r : x0 - r;
-  *tau = r > 0.0 ? 1.0 / (r * (r + fabs(x0))) : 0.0;
-}
-
-// The same with about 44 correct bits before the final rounding, in pairs of
-// floats (Dekker 1971: residuals of a square root, a sum and a product are
-// exact or nearly so with fma).
-__device__ __forceinline__ void reflector(float r2, float x0, float* head, float* tau) {
-  const float r = sqrtf(r2);
-  if (!(r > 0.f)) {
-    *head = x0;
-    *tau = 0.f;
-    return;
-  }
-  const float rl = fmaf(-r, r, r2) / (2.f * r);  // sqrt(r2) = r + rl
-  const float a = fabsf(x0);
-  const float h = r + a, t = h - r;                      // r + |x0| = h + hl
-  const float hl = ((r - (h - t)) + (a - t)) + rl;
-  const float q = r * h;                                 // r (r + |x0|) = q + ql
-  const float ql = fmaf(r, h, -q) + fmaf(r, hl, rl * h);
-  const float t0 = 1.f / q;
-  *tau = fmaf(t0, fmaf(-q, t0, 1.f) - ql * t0, t0);
-  *head = copysignf(h + hl, x0 >= 0.f ? 1.f : -1.f);
-}
-
 template <typename real>
 struct Exchange {
   real val;        // largest local squared norm
@@ -304,7 +275,7 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const int* __restrict__ or
     const real* ocol = cl.map_shared_rank(Gs, owner) + (int64_t)oloc * ldsm;
     const real x0 = ocol[j];
     real head, tj;
-    reflector(r2, x0, &head, &tj);
+    householder_scalars(r2, x0, &head, &tj);
     for (int i = j + threadIdx.x; i < m; i += blockDim.x) {
       const real v = (i == j) ? head : ocol[i];
       vloc[i] = v;
@@ -550,7 +521,7 @@ qr_reg_kernel(const PrepTask* __restrict__ tasks, const int* __restrict__ order,
       const real r2 = __shfl_sync(0xffffffffu, used ? real(-1) : nrm, src);
       __syncwarp();
       real head, tau;
-      reflector(r2, x0, &head, &tau);
+      householder_scalars(r2, x0, &head, &tau);
       if (lane == 0) {
         vs[par][(j % TPC) * kLdv + j / TPC] = head;
         vs[par][kInfo] = r2;
