@@ -183,7 +183,19 @@ struct SchurTask {
   int64_t P, Q;     // factor offsets of the P/Q storages
   int64_t map;      // offset of the neighbour runs (Seg list, nb entries)
   int64_t base;     // offset into the block-base table (nb*nb entries)
-  int64_t ldn;      // offset into the neighbour-ld array (nb entries)
+  int64_t nbr;      // offset into the neighbour list (nb entries)
+};
+
+// A neighbour of a Schur task: its cluster and its blocks' leading dimension.
+struct SchurNbr {
+  int id, ld;
+};
+
+// The block pattern of a level on the device: columns of cluster i's row in
+// col[ptr[i] .. ptr[i + 1]) (ascending), block offsets in off.
+struct DevPattern {
+  const int *ptr, *col;
+  const int64_t* off;
 };
 
 // Scatter of coarse rows/columns into the blocks after a cluster step.
@@ -231,8 +243,12 @@ size_t dense_top_tc_scratch(int n);
 // Schur-complement update of a colour class (the SIMT schur launch's
 // arguments) with tensor-core products in the given mode.
 void schur_tc(int mode, const SchurTask* tasks, int ntask, int maxnw, const float* fac,
-              float* arena, const Seg* segs, const int64_t* base, const int* ldn, const int* rank,
-              DevError* err, cudaStream_t st);
+              float* arena, const Seg* segs, const int64_t* base, const SchurNbr* nbr,
+              const int* rank, DevError* err, cudaStream_t st);
+// The target blocks of every pair of a task's neighbours (the block-base
+// table) from the level's pattern.
+void schur_targets(const SchurTask* tasks, int ntask, int maxnb, const SchurNbr* nbr,
+                   const DevPattern& P, int64_t* base, DevError* err, cudaStream_t st);
 void dense_top_tc(float* A, int64_t lda, int n, float* X, float* W, DevError* err, int level,
                   cudaStream_t st);
 
@@ -276,7 +292,7 @@ struct Launch {
                           const Seg* segs, const int* rank,
                           cudaStream_t st);
   static void schur(const SchurTask* tasks_dev, int ntask, int maxnw, const real* fac,
-                    real* arena, const Seg* segs, const int64_t* base, const int* ldn,
+                    real* arena, const Seg* segs, const int64_t* base, const SchurNbr* nbr,
                     const int* rank, cudaStream_t st);
   static void scatter(const ScatterSeg* segs_dev, int nseg, int maxw, const real* src,
                       real* arena, const int* rank, cudaStream_t st);

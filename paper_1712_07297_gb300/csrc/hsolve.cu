@@ -220,6 +220,7 @@ struct hsolve_handle {
   // scratch
   DevBuf d_err;
   DevBuf ws, wsd, blob_dev, blob2, blob3, cnt;
+  DevBuf sbase;  // target blocks of a class's Schur updates
   DevBuf top_w;  // scratch of the tensor-core dense top
   PinnedBuf pin, pin2, pin3;
   PinnedBuf pin_rank;  // ranks and error words copied back class by class
@@ -509,27 +510,23 @@ struct HostTimer {
   }
 };
 
-void check_dev_error(hsolve_handle* h) {
-  DevError e{};
-  HS_CUDA(cudaMemcpyAsync(&e, h->d_err.p, sizeof(DevError), cudaMemcpyDeviceToHost, h->st));
-  HS_CUDA(cudaStreamSynchronize(h->st));
-  if (e.code != 0) {
-    throw Fail((hsolve_status)e.code, std::string(e.code == HSOLVE_ERR_NOT_SPD
-                                                      ? "Cholesky pivot not positive"
-                                                      : "zero pivot in LU") +
-                                          " at level " + std::to_string(e.level) +
-                                          ", cluster " + std::to_string(e.cluster));
-  }
-}
-
 // A copy of the device error word taken behind a class's kernels.
 void check_err_copy(const DevError& e) {
   if (e.code != 0)
     throw Fail((hsolve_status)e.code, std::string(e.code == HSOLVE_ERR_NOT_SPD
                                                       ? "Cholesky pivot not positive"
-                                                      : "zero pivot in LU") +
+                                                      : e.code == HSOLVE_ERR_CUDA
+                                                            ? "internal: missing Schur target block"
+                                                            : "zero pivot in LU") +
                                           " at level " + std::to_string(e.level) +
                                           ", cluster " + std::to_string(e.cluster));
+}
+
+void check_dev_error(hsolve_handle* h) {
+  DevError e{};
+  HS_CUDA(cudaMemcpyAsync(&e, h->d_err.p, sizeof(DevError), cudaMemcpyDeviceToHost, h->st));
+  HS_CUDA(cudaStreamSynchronize(h->st));
+  check_err_copy(e);
 }
 
 // ---------------------------------------------------------------------------
@@ -628,48 +625,39 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
   FL.cls.clear();
   // rank-independent part of every cluster's tasks, built in parallel for
   // the whole level: its pattern row without the diagonal (neighbour or fill
-  // block, both block offsets) and, for every ordered pair of its
-  // neighbours, the offset of their block (the Schur-complement targets)
+  // block, both block offsets)
   struct NbPre {
     int j, kind;
     int64_t p_sj, p_js;
   };
   std::vector<std::vector<NbPre>> pre_nb(nc);
-  std::vector<std::vector<int64_t>> pre_sb(nc);
-  // The pair table walks each neighbour's pattern row once against a
-  // per-thread map cluster -> neighbour index (reset after every cluster)
-  // instead of searching the row for every pair.
-  auto prepass = [&](int s) {
-    thread_local std::vector<int> pos;
-    if ((int)pos.size() < nc) pos.assign(nc, -1);
-    auto& L = pre_nb[s];
-    L.clear();
-    L.reserve(P.ptr[s + 1] - P.ptr[s]);
-    int nn = 0;
-    for (int p = P.ptr[s]; p < P.ptr[s + 1]; p++) {
-      const int j = P.col[p];
-      if (j == s) continue;
-      L.push_back({j, (int)P.kind[p], P.off[p], P.off[P.find(j, s)]});
-      if (P.kind[p] == 1) pos[j] = nn++;
-    }
-    auto& sb = pre_sb[s];
-    sb.assign((size_t)nn * nn, -1);
-    for (auto& ea : L) {
-      if (ea.kind != 1) continue;
-      int64_t* row = sb.data() + (size_t)pos[ea.j] * nn;
-      for (int q = P.ptr[ea.j]; q < P.ptr[ea.j + 1]; q++) {
-        const int b = pos[P.col[q]];
-        if (b >= 0) row[b] = P.off[q];
-      }
-    }
-    for (auto& ea : L)
-      if (ea.kind == 1) pos[ea.j] = -1;
-  };
   {
     HostTimer ht(h, "host.prepass");
     parallel_for(nc, [&](int s) {
-      if (P.m[s] > 0) prepass(s);
+      if (P.m[s] == 0) return;
+      auto& L = pre_nb[s];
+      L.reserve(P.ptr[s + 1] - P.ptr[s]);
+      for (int p = P.ptr[s]; p < P.ptr[s + 1]; p++)
+        if (P.col[p] != s)
+          L.push_back({P.col[p], (int)P.kind[p], P.off[p], P.off[P.find(P.col[p], s)]});
     });
+  }
+  // the pattern on the device: the Schur updates' target blocks are found there
+  DevBuf d_pat;
+  DevPattern dpat{};
+  {
+    HostTimer ht(h, "host.pattern");
+    const size_t ne = P.col.size(), po = (sizeof(int64_t) * ne + 15) / 16 * 16,
+                 pc = po + (sizeof(int) * ne + 15) / 16 * 16;
+    d_pat.alloc(pc + sizeof(int) * (nc + 1));
+    char* d = d_pat.as<char>();
+    HS_CUDA(cudaMemcpyAsync(d, P.off.data(), sizeof(int64_t) * ne, cudaMemcpyHostToDevice, h->st));
+    HS_CUDA(cudaMemcpyAsync(d + po, P.col.data(), sizeof(int) * ne, cudaMemcpyHostToDevice, h->st));
+    HS_CUDA(cudaMemcpyAsync(d + pc, P.ptr.data(), sizeof(int) * (nc + 1), cudaMemcpyHostToDevice,
+                            h->st));
+    dpat.off = reinterpret_cast<const int64_t*>(d);
+    dpat.col = reinterpret_cast<const int*>(d + po);
+    dpat.ptr = reinterpret_cast<const int*>(d + pc);
   }
   // a single large cluster (the dense top of Alg. 1) goes to the blocked
   // multi-CTA Cholesky (SPD) or LU with partial pivoting (general) and the
@@ -722,10 +710,10 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     h->factor_flops += fl;
     h->apply_bytes += (int64_t)sizeof(real) * 2 * ((int64_t)n * n + 2 * (int64_t)n);
   }
-  struct Nb { int j, w; int64_t p_sj, p_js; int ia; };
+  struct Nb { int j, w; int64_t p_sj, p_js; };
   // Every cluster's tasks are built in parallel with offsets relative to the
   // cluster (its gathered-column runs, workspace, norms workspace, Schur
-  // block bases and neighbour lds, vector-map entries), then concatenated in
+  // neighbours, vector-map entries), then concatenated in
   // cluster order with the offsets rebased.
   struct ClusterBuild {
     PrepTask pt;
@@ -734,13 +722,11 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     SchurTask sc;
     bool has_sk = false, has_Y = false, has_E = false, has_sc = false;
     std::vector<Seg> segs;
-    std::vector<int64_t> sbase;
-    std::vector<int> sld;
+    std::vector<SchurNbr> snb;
     std::vector<ScatterSeg> segN, segW;
     std::vector<std::pair<int, int>> nbs;  // neighbours (id, width), column order
     int64_t ws = 0, wsd = 0;
     int nw = 0, nwf = 0, maxw = 0;
-    bool bad = false;
   };
   std::vector<ClusterBuild> cbs_keep;
   // The classes run as a pipeline between host and device: a class's ranks
@@ -760,13 +746,12 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     std::vector<SchurTask> sch;
     std::vector<ScatterSeg> segN, segW;
     std::vector<Seg> segs;
-    std::vector<int64_t> sbase;
-    std::vector<int> sld;
-    int64_t ws_e = 0, wsd_e = 0;
-    int maxm = 0, maxnw = 0, maxnwf = 0, maxw_seg = 0;
+    std::vector<SchurNbr> snb;
+    int64_t ws_e = 0, wsd_e = 0, base_e = 0;
+    int maxm = 0, maxnw = 0, maxnwf = 0, maxw_seg = 0, maxnb = 0;
     Blob b;
     size_t o_sk = 0, o_prep = 0, o_gY = 0, o_gXT = 0, o_gE = 0, o_gE2 = 0, o_sch = 0,
-           o_segN = 0, o_segW = 0, o_segs = 0, o_sbase = 0, o_sld = 0;
+           o_segN = 0, o_segW = 0, o_segs = 0, o_snb = 0;
   };
   // Tasks of the first class at or after c with clusters left; false when
   // no class is left.
@@ -791,8 +776,7 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     std::vector<SchurTask>& sch = T.sch;
     std::vector<ScatterSeg>&segN = T.segN, &segW = T.segW;
     std::vector<Seg>& segs = T.segs;
-    std::vector<int64_t>& sbase = T.sbase;
-    std::vector<int>& sld = T.sld;
+    std::vector<SchurNbr>& snb = T.snb;
     int64_t &ws_e = T.ws_e, &wsd_e = T.wsd_e;
     int &maxm = T.maxm, &maxnw = T.maxnw, &maxnwf = T.maxnwf, &maxw_seg = T.maxw_seg;
     sk.clear();
@@ -804,24 +788,22 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     segN.clear();
     segW.clear();
     segs.clear();
-    sbase.clear();
-    sld.clear();
+    snb.clear();
     maxl = 0;
-    ws_e = wsd_e = 0;
-    maxm = maxnw = maxnwf = maxw_seg = 0;
+    ws_e = wsd_e = T.base_e = 0;
+    maxm = maxnw = maxnwf = maxw_seg = T.maxnb = 0;
     // Every cluster's tasks are built in parallel with offsets relative to
     // the cluster (its gathered-column runs, workspace, norms workspace,
-    // Schur block bases and neighbour lds, vector-map entries), then
+    // Schur neighbours, vector-map entries), then
     // concatenated in cluster order with the offsets rebased.
     if ((int)cbs_keep.size() < nt) cbs_keep.resize(nt);
     std::vector<ClusterBuild>& cbs = cbs_keep;  // kept across classes (capacities reused)
     std::unique_ptr<HostTimer> hpar(new HostTimer(h, "host.b_par"));
     parallel_for(nt, [&](int t) {
       ClusterBuild& cb = cbs[t];
-      cb.has_sk = cb.has_Y = cb.has_E = cb.has_sc = cb.bad = false;
+      cb.has_sk = cb.has_Y = cb.has_E = cb.has_sc = false;
       cb.segs.clear();
-      cb.sbase.clear();
-      cb.sld.clear();
+      cb.snb.clear();
       cb.segN.clear();
       cb.segW.clear();
       cb.nbs.clear();
@@ -829,11 +811,9 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
       const int s = S[t];
       const int m = cur[s];
       std::vector<Nb> N, W;
-      int nn_all = 0;  // neighbours in the pattern (index base of pre_sb)
       for (auto& e0 : pre_nb[s]) {
-        const int ia = e0.kind == 1 ? nn_all++ : -1;
         if (cur[e0.j] == 0) continue;
-        Nb e{e0.j, cur[e0.j], e0.p_sj, e0.p_js, ia};
+        Nb e{e0.j, cur[e0.j], e0.p_sj, e0.p_js};
         if (e0.kind == 1) N.push_back(e);
         else W.push_back(e);
       }
@@ -962,23 +942,15 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
         cb.maxw = std::max(cb.maxw, e.w);
         c0 += e.w;
       }
-      // Schur task: maps and block bases
+      // Schur task: the A_sN runs and the neighbours
       if (nw > 0) {
         SchurTask sc{};
         sc.s = s; sc.m = m; sc.nw = nw; sc.nb = (int)N.size();
         sc.P = sym ? oY[s] : oXT[s];
         sc.Q = oY[s];
         sc.map = ncol0;  // the A_sN runs: one per neighbour, colstart = its offset
-        sc.base = 0;
-        const auto& sb = pre_sb[s];
-        for (int a = 0; a < (int)N.size(); a++)
-          for (int b = 0; b < (int)N.size(); b++) {
-            const int64_t o = sb[(size_t)N[a].ia * nn_all + N[b].ia];
-            if (o < 0) cb.bad = true;
-            cb.sbase.push_back(o);
-          }
-        sc.ldn = 0;
-        for (auto& e : N) cb.sld.push_back(P.ld[e.j]);
+        sc.base = sc.nbr = 0;
+        for (auto& e : N) cb.snb.push_back({e.j, P.ld[e.j]});
         cb.sc = sc;
         cb.has_sc = true;
       }
@@ -988,7 +960,6 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     std::unique_ptr<HostTimer> hmerge(new HostTimer(h, "host.b_merge"));
     for (int t = 0; t < nt; t++) {
       ClusterBuild& cb = cbs[t];
-      if (cb.bad) throw Fail(HSOLVE_ERR_CUDA, "internal: missing Schur target block");
       const int s = S[t];
       const int m = cur[s];
       maxm = std::max(maxm, m);
@@ -1046,10 +1017,11 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
       if (cb.has_sc) {
         SchurTask sc = cb.sc;
         sc.map += sg0;
-        sc.base = (int64_t)sbase.size();
-        sc.ldn = (int64_t)sld.size();
-        sbase.insert(sbase.end(), cb.sbase.begin(), cb.sbase.end());
-        sld.insert(sld.end(), cb.sld.begin(), cb.sld.end());
+        sc.nbr = (int64_t)snb.size();
+        sc.base = T.base_e;
+        T.base_e += (int64_t)sc.nb * sc.nb;
+        T.maxnb = std::max(T.maxnb, sc.nb);
+        snb.insert(snb.end(), cb.snb.begin(), cb.snb.end());
         sch.push_back(sc);
       }
       segs.insert(segs.end(), cb.segs.begin(), cb.segs.end());
@@ -1081,8 +1053,7 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     T.o_segN = b.add(segN);
     T.o_segW = b.add(segW);
     T.o_segs = b.add(segs);
-    T.o_sbase = b.add(sbase);
-    T.o_sld = b.add(sld);
+    T.o_snb = b.add(snb);
     return true;
   };
   h->pin_rank.ensure(sizeof(int) * std::max(nc, 1) + 2 * sizeof(DevError));
@@ -1113,9 +1084,10 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     const int maxm = T.maxm, maxnw = T.maxnw, maxnwf = T.maxnwf, maxw_seg = T.maxw_seg;
     const size_t o_sk = T.o_sk, o_prep = T.o_prep, o_gY = T.o_gY, o_gXT = T.o_gXT,
                  o_gE = T.o_gE, o_gE2 = T.o_gE2, o_sch = T.o_sch, o_segN = T.o_segN,
-                 o_segW = T.o_segW, o_segs = T.o_segs, o_sbase = T.o_sbase, o_sld = T.o_sld;
+                 o_segW = T.o_segW, o_segs = T.o_segs, o_snb = T.o_snb;
     h->ws.ensure(std::max<int64_t>(T.ws_e, 4) * sizeof(real));
     h->wsd.ensure(std::max<int64_t>(T.wsd_e, 4) * sizeof(double));
+    h->sbase.ensure(std::max<int64_t>(T.base_e, 2) * sizeof(int64_t));
     char* d = upload_blob(h, T.b);
     // the ranks are final after the pivoted QR: in the cluster-QR kernel,
     // unless some cluster's QR runs inside the per-cluster kernel
@@ -1298,18 +1270,19 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
       Launch<real>::scatter(reinterpret_cast<const ScatterSeg*>(d + o_segW), (int)segW.size(),
                             maxw_seg, ws, arena, rank, h->st);
     });
-    timed_lv(h, "schur", level, 1, [&] {
+    timed_lv(h, "schur", level, 2, [&] {
       const int tm = tc_schur_mode(h->prec);
+      const SchurNbr* d_snb = reinterpret_cast<const SchurNbr*>(d + o_snb);
+      int64_t* base = h->sbase.as<int64_t>();
+      schur_targets(reinterpret_cast<const SchurTask*>(d + o_sch), (int)sch.size(), T.maxnb, d_snb,
+                    dpat, base, h->d_err.as<DevError>(), h->st);
       if (std::is_same<real, float>::value && tm >= 0)
         schur_tc(tm, reinterpret_cast<const SchurTask*>(d + o_sch), (int)sch.size(), maxnw,
                  reinterpret_cast<const float*>(fac), reinterpret_cast<float*>(arena), d_segs,
-                 reinterpret_cast<const int64_t*>(d + o_sbase),
-                 reinterpret_cast<const int*>(d + o_sld), rank, h->d_err.as<DevError>(), h->st);
+                 base, d_snb, rank, h->d_err.as<DevError>(), h->st);
       else
         Launch<real>::schur(reinterpret_cast<const SchurTask*>(d + o_sch), (int)sch.size(),
-                            maxnw, fac, arena, d_segs,
-                            reinterpret_cast<const int64_t*>(d + o_sbase),
-                            reinterpret_cast<const int*>(d + o_sld), rank, h->st);
+                            maxnw, fac, arena, d_segs, base, d_snb, rank, h->st);
     });
     if (!rank_copied) copy_ranks();
     // the error word behind this class's kernels (read one class later)

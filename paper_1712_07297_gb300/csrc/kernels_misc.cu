@@ -196,7 +196,7 @@ template <typename real>
 __global__ void __launch_bounds__(256)
 schur_kernel(const SchurTask* __restrict__ tasks, const real* __restrict__ fac,
              real* __restrict__ arena, const Seg* __restrict__ segs,
-             const int64_t* __restrict__ base, const int* __restrict__ ldn,
+             const int64_t* __restrict__ base, const SchurNbr* __restrict__ nbr,
              const int* __restrict__ rank) {
   const SchurTask tk = tasks[blockIdx.z];
   const int k = rank[tk.s];
@@ -281,12 +281,12 @@ schur_kernel(const SchurTask* __restrict__ tasks, const real* __restrict__ fac,
   // read-modify-write of the target blocks from the staged tile, consecutive
   // threads on consecutive rows of a block (column-major: contiguous)
   const int64_t* bs = base + tk.base;
-  const int* ldv = ldn + tk.ldn;
+  const SchurNbr* nb = nbr + tk.nbr;
   for (int e = threadIdx.x; e < TM * TN; e += blockDim.x) {
     const int ii = e % TM, jj = e / TM, gi = i0 + ii, gj = j0 + jj;
     if (gi >= N || gj >= N || (sym && gj > gi)) continue;
     const int a = rblk[ii];
-    arena[bs[a * tk.nb + cblk[jj]] + rloc[ii] + (int64_t)cloc[jj] * ldv[a]] -= Cs[jj][ii];
+    arena[bs[a * tk.nb + cblk[jj]] + rloc[ii] + (int64_t)cloc[jj] * nb[a].ld] -= Cs[jj][ii];
   }
   if (!sym) return;
   // the mirror elements (c, r) of the strictly lower part: row gj of block
@@ -295,7 +295,35 @@ schur_kernel(const SchurTask* __restrict__ tasks, const real* __restrict__ fac,
     const int jj = e % TN, ii = e / TN, gi = i0 + ii, gj = j0 + jj;
     if (gi >= N || gj >= gi) continue;
     const int b = cblk[jj];
-    arena[bs[b * tk.nb + rblk[ii]] + cloc[jj] + (int64_t)rloc[ii] * ldv[b]] -= Cs[jj][ii];
+    arena[bs[b * tk.nb + rblk[ii]] + cloc[jj] + (int64_t)rloc[ii] * nb[b].ld] -= Cs[jj][ii];
+  }
+}
+
+// base[a * nb + b] = arena offset of block (neighbour a, neighbour b) of every
+// task, one thread per pair, by bisection of the pattern row.  (The host built
+// and uploaded this table: 124 of 170 ms of its work per factorization of 96^3
+// went into it; here it takes about 4 us per class.  Looking the blocks up in
+// the Schur update itself put the searches in front of every tile: 140 to 160
+// ms of updates at 96^3 against 132.)
+__global__ void schur_targets_kernel(const SchurTask* __restrict__ tasks,
+                                     const SchurNbr* __restrict__ nbr, DevPattern P,
+                                     int64_t* __restrict__ base, DevError* err) {
+  const SchurTask tk = tasks[blockIdx.y];
+  const SchurNbr* nb = nbr + tk.nbr;
+  const int n = tk.nb * tk.nb;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int i = nb[e / tk.nb].id, j = nb[e % tk.nb].id;
+    int lo = P.ptr[i], hi = P.ptr[i + 1];
+    const int end = hi;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (P.col[mid] < j) lo = mid + 1;
+      else hi = mid;
+    }
+    const bool have = lo < end && P.col[lo] == j;
+    // two neighbours of a cluster are within distance two: the block exists
+    if (!have && atomicCAS(&err->code, 0, (int)HSOLVE_ERR_CUDA) == 0) err->cluster = tk.s;
+    base[tk.base + e] = have ? P.off[lo] : 0;
   }
 }
 
@@ -531,13 +559,24 @@ void Launch<real>::sketch(const SketchTask* tasks_dev, int ntask, int maxm, int 
 
 template <typename real>
 void Launch<real>::schur(const SchurTask* tasks_dev, int ntask, int maxnw, const real* fac,
-                         real* arena, const Seg* segs, const int64_t* base, const int* ldn,
+                         real* arena, const Seg* segs, const int64_t* base, const SchurNbr* nbr,
                          const int* rank, cudaStream_t st) {
   if (ntask <= 0 || maxnw <= 0) return;
   for (int t0 = 0; t0 < ntask; t0 += kMaxGridYZ) {
     dim3 grid((maxnw + TN - 1) / TN, (maxnw + TM - 1) / TM, std::min(kMaxGridYZ, ntask - t0));
     count_launch();
-    schur_kernel<real><<<grid, 256, 0, st>>>(tasks_dev + t0, fac, arena, segs, base, ldn, rank);
+    schur_kernel<real><<<grid, 256, 0, st>>>(tasks_dev + t0, fac, arena, segs, base, nbr, rank);
+  }
+}
+
+void schur_targets(const SchurTask* tasks, int ntask, int maxnb, const SchurNbr* nbr,
+                   const DevPattern& P, int64_t* base, DevError* err, cudaStream_t st) {
+  if (ntask <= 0 || maxnb <= 0) return;
+  for (int t0 = 0; t0 < ntask; t0 += kMaxGridYZ) {
+    const int64_t pairs = (int64_t)maxnb * maxnb;
+    dim3 grid((int)std::min<int64_t>(128, (pairs + 255) / 256), std::min(kMaxGridYZ, ntask - t0));
+    count_launch();
+    schur_targets_kernel<<<grid, 256, 0, st>>>(tasks + t0, nbr, P, base, err);
   }
 }
 

@@ -378,7 +378,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kTcThreads)
 schur_tc_kernel(const SchurTask* __restrict__ tasks, const float* __restrict__ fac,
                 float* __restrict__ arena, const Seg* __restrict__ segs,
-                const int64_t* __restrict__ base, const int* __restrict__ ldn,
+                const int64_t* __restrict__ base, const SchurNbr* __restrict__ nbr,
                 const int* __restrict__ rank, DevError* err) {
   using MD = TcMode<MODE>;
   const SchurTask tk = tasks[blockIdx.z];
@@ -476,9 +476,9 @@ schur_tc_kernel(const SchurTask* __restrict__ tasks, const float* __restrict__ f
     const int ii = warp * 32 + lane, gi = i0 + ii;
     const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
     const int64_t* bs = base + tk.base;
-    const int* ldv = ldn + tk.ldn;
+    const SchurNbr* nb = nbr + tk.nbr;
     const int a = rblk[ii], lr = rloc[ii];
-    const int64_t lda = ldv[a];
+    const int64_t lda = nb[a].ld;
     for (int jc = 0; jc < TN; jc += 32) {
       float v[32];
       tmem_ld32(tl + jc, v);
@@ -728,7 +728,7 @@ void tc_gemm(int mode, int M, int N, int K, const float* A, int64_t rsa, int64_t
 
 template <int MODE>
 void launch_schur(const SchurTask* tasks, int ntask, int maxnw, const float* fac, float* arena,
-                  const Seg* segs, const int64_t* base, const int* ldn, const int* rank,
+                  const Seg* segs, const int64_t* base, const SchurNbr* nbr, const int* rank,
                   DevError* err, cudaStream_t st) {
   const size_t smem = 2 * TcMode<MODE>::kStageBytes + 1024;
   static const bool attr_set = [smem] {
@@ -740,21 +740,21 @@ void launch_schur(const SchurTask* tasks, int ntask, int maxnw, const float* fac
   for (int t0 = 0; t0 < ntask; t0 += 65535) {
     dim3 grid((maxnw + TN - 1) / TN, (maxnw + TM - 1) / TM, std::min(65535, ntask - t0));
     count_launch();
-    schur_tc_kernel<MODE><<<grid, kTcThreads, smem, st>>>(tasks + t0, fac, arena, segs, base, ldn,
+    schur_tc_kernel<MODE><<<grid, kTcThreads, smem, st>>>(tasks + t0, fac, arena, segs, base, nbr,
                                                           rank, err);
   }
 }
 
 void schur_tc(int mode, const SchurTask* tasks, int ntask, int maxnw, const float* fac,
-              float* arena, const Seg* segs, const int64_t* base, const int* ldn, const int* rank,
+              float* arena, const Seg* segs, const int64_t* base, const SchurNbr* nbr, const int* rank,
               DevError* err, cudaStream_t st) {
   if (ntask <= 0 || maxnw <= 0) return;
   if (mode == 0)
-    launch_schur<0>(tasks, ntask, maxnw, fac, arena, segs, base, ldn, rank, err, st);
+    launch_schur<0>(tasks, ntask, maxnw, fac, arena, segs, base, nbr, rank, err, st);
   else if (mode == 1)
-    launch_schur<1>(tasks, ntask, maxnw, fac, arena, segs, base, ldn, rank, err, st);
+    launch_schur<1>(tasks, ntask, maxnw, fac, arena, segs, base, nbr, rank, err, st);
   else
-    launch_schur<2>(tasks, ntask, maxnw, fac, arena, segs, base, ldn, rank, err, st);
+    launch_schur<2>(tasks, ntask, maxnw, fac, arena, segs, base, nbr, rank, err, st);
 }
 
 size_t dense_top_tc_scratch(int n) { return (size_t)(n / 2 + kLeaf) * (size_t)(n / 2 + kLeaf); }
