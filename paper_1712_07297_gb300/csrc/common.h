@@ -294,7 +294,7 @@ struct Launch {
   static void schur(const SchurTask* tasks_dev, int ntask, int maxnw, const real* fac,
                     real* arena, const Seg* segs, const int64_t* base, const SchurNbr* nbr,
                     const int* rank, cudaStream_t st);
-  static void scatter(const ScatterSeg* segs_dev, int nseg, int maxw, const real* src,
+  static void scatter(const ScatterSeg* segs_dev, int nseg, int maxw, int maxm, const real* src,
                       real* arena, const int* rank, cudaStream_t st);
   static void copy_blocks(const CopyTask* tasks_dev, int ntask, const real* src, real* dst,
                           cudaStream_t st);

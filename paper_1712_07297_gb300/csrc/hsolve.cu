@@ -1266,9 +1266,9 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     });
     timed_lv(h, "scatter", level, 2, [&] {
       Launch<real>::scatter(reinterpret_cast<const ScatterSeg*>(d + o_segN), (int)segN.size(),
-                            maxw_seg, fac, arena, rank, h->st);
+                            maxw_seg, maxm, fac, arena, rank, h->st);
       Launch<real>::scatter(reinterpret_cast<const ScatterSeg*>(d + o_segW), (int)segW.size(),
-                            maxw_seg, ws, arena, rank, h->st);
+                            maxw_seg, maxm, ws, arena, rank, h->st);
     });
     timed_lv(h, "schur", level, 2, [&] {
       const int tm = tc_schur_mode(h->prec);
