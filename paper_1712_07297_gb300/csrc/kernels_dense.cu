@@ -29,12 +29,12 @@ struct PrepThreads {
   static constexpr int value = sizeof(real) == 4 ? 512 : 256;
 };
 constexpr double kPivotTieRtol = 1e-10;  // LU pivot search
+constexpr int kRowsMax = 256;  // triangular inverses with columns or rows in registers
 // near-ties of the column-pivoted QR, relative: 1e-10 in float64; float32
 // squared norms carry ~1e-7 relative rounding, so ties of exact arithmetic
 // are recognised within 1e-5
 template <typename real>
 __device__ __forceinline__ double qr_tie_rtol() { return sizeof(real) == 8 ? 1e-10 : 1e-5; }
-constexpr int GT = 64, GK = 16;  // CTA GEMM tile and inner chunk
 
 template <typename real>
 __device__ __forceinline__ real sqrt_(real x);
@@ -43,81 +43,56 @@ __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
 template <>
 __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
 
-// C (M x N, ldc) = alpha * op(A) * op(B) + beta * C, whole CTA (NT =
-// PrepThreads threads, 64 x 64 output tiles, GR x 4 outputs per thread with
-// GR = 1024 / NT, inner chunks of 16 staged in shared memory `sh` of
-// 2 * 16 * 65 reals).  C must not alias A or B.
+// C (M x N, ldc) = op(A) * op(B), whole CTA, RM x RN outputs per thread straight
+// from the operands (shared memory, or the workspace through L1); the sum over l
+// runs in ascending order in one accumulator.  A thread's rows are strided so
+// that a warp reads consecutive ones.  C must not alias A or B.  (Staging 16
+// inner indices at a time instead took two barriers per chunk: 43 us for the
+// 128 x 128 x 128 product of [U V]^T A_ss^{-1} against 17.)
+template <typename real, int RM, int RN>
+__device__ __forceinline__ void gemm_tiles(int M, int N, int K, const real* A, int ars, int acs,
+                                           const real* B, int brs, int bcs, real* C, int ldc) {
+  const int nti = (M + RM - 1) / RM, n = nti * ((N + RN - 1) / RN);
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int ti = t % nti, jf = t / nti * RN;
+    int ao[RM], bo[RN];
+#pragma unroll
+    for (int r = 0; r < RM; r++) ao[r] = min(ti + r * nti, M - 1) * ars;
+#pragma unroll
+    for (int c = 0; c < RN; c++) bo[c] = min(jf + c, N - 1) * bcs;
+    real acc[RM][RN];
+#pragma unroll
+    for (int r = 0; r < RM; r++)
+#pragma unroll
+      for (int c = 0; c < RN; c++) acc[r][c] = 0;
+#pragma unroll 4
+    for (int l = 0; l < K; l++) {
+      real a[RM], b[RN];
+#pragma unroll
+      for (int r = 0; r < RM; r++) a[r] = A[ao[r] + l * acs];
+#pragma unroll
+      for (int c = 0; c < RN; c++) b[c] = B[bo[c] + l * brs];
+#pragma unroll
+      for (int r = 0; r < RM; r++)
+#pragma unroll
+        for (int c = 0; c < RN; c++) acc[r][c] += a[r] * b[c];
+    }
+#pragma unroll
+    for (int r = 0; r < RM; r++)
+#pragma unroll
+      for (int c = 0; c < RN; c++)
+        if (ti + r * nti < M && jf + c < N) C[ti + r * nti + (int64_t)(jf + c) * ldc] = acc[r][c];
+  }
+}
+
 template <typename real>
 __device__ void cta_gemm(int M, int N, int K, const real* A, int lda, bool ta, const real* B,
-                         int ldb, bool tb, real* C, int ldc, real alpha, real beta, real* sh) {
-  constexpr int NT = PrepThreads<real>::value;
-  constexpr int GR = 1024 / NT, RS = NT / 16;  // rows per thread, row stride
-  real* As = sh;
-  real* Bs = sh + GK * (GT + 1);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  for (int i0 = 0; i0 < M; i0 += GT)
-    for (int j0 = 0; j0 < N; j0 += GT) {
-      real acc[GR][4];
-#pragma unroll
-      for (int p = 0; p < GR; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc[p][q] = 0;
-      for (int l0 = 0; l0 < K; l0 += GK) {
-        for (int e = threadIdx.x; e < GT * GK; e += blockDim.x) {
-          int i, l;
-          if (!ta) {
-            i = e % GT;
-            l = e / GT;
-          } else {
-            l = e % GK;
-            i = e / GK;
-          }
-          int gi = i0 + i, gl = l0 + l;
-          real v = 0;
-          if (gi < M && gl < K) v = ta ? A[gl + (int64_t)gi * lda] : A[gi + (int64_t)gl * lda];
-          As[l * (GT + 1) + i] = v;
-        }
-        for (int e = threadIdx.x; e < GT * GK; e += blockDim.x) {
-          int l, j;
-          if (!tb) {
-            l = e % GK;
-            j = e / GK;
-          } else {
-            j = e % GT;
-            l = e / GT;
-          }
-          int gl = l0 + l, gj = j0 + j;
-          real v = 0;
-          if (gl < K && gj < N) v = tb ? B[gj + (int64_t)gl * ldb] : B[gl + (int64_t)gj * ldb];
-          Bs[l * (GT + 1) + j] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int l = 0; l < GK; l++) {
-          real a[GR], b[4];
-#pragma unroll
-          for (int p = 0; p < GR; p++) a[p] = As[l * (GT + 1) + ty + RS * p];
-#pragma unroll
-          for (int q = 0; q < 4; q++) b[q] = Bs[l * (GT + 1) + tx + 16 * q];
-#pragma unroll
-          for (int p = 0; p < GR; p++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[p][q] += a[p] * b[q];
-        }
-        __syncthreads();
-      }
-#pragma unroll
-      for (int p = 0; p < GR; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          int gi = i0 + ty + RS * p, gj = j0 + tx + 16 * q;
-          if (gi < M && gj < N) {
-            real c = alpha * acc[p][q];
-            if (beta != real(0)) c += beta * C[gi + (int64_t)gj * ldc];
-            C[gi + (int64_t)gj * ldc] = c;
-          }
-        }
-    }
+                         int ldb, bool tb, real* C, int ldc) {
+  const int ars = ta ? lda : 1, acs = ta ? 1 : lda, brs = tb ? ldb : 1, bcs = tb ? 1 : ldb;
+  if (M * N >= 12 * (int)blockDim.x)
+    gemm_tiles<real, 4, 4>(M, N, K, A, ars, acs, B, brs, bcs, C, ldc);
+  else
+    gemm_tiles<real, 2, 2>(M, N, K, A, ars, acs, B, brs, bcs, C, ldc);
   __syncthreads();
 }
 
@@ -194,49 +169,197 @@ __device__ bool cta_cholesky(int n, real* A, int lda, int* sflag) {
   return true;
 }
 
-// In-place LU with partial pivoting, P A = L U (unit lower L).  piv[j] = row
-// swapped with j at step j.  Near-ties (|a| >= (1 - 1e-10) max) go to the
-// lowest row.  Returns false for an exactly zero pivot column.
 __device__ double cta_max_d(double v, double* red);
 __device__ int cta_min_i(int v, int* red);
 
+// One warp: the pivot row of column c at or below row j -- the largest
+// magnitude, near-ties (|a| >= (1 - 1e-10) max, in float32 equal magnitudes) to
+// the lowest row; -1 for a zero column.
+__device__ __forceinline__ int warp_pivot(int n, int j, const float* c) {
+  unsigned mx = 0;
+  for (int i = j + lane_id(); i < n; i += 32) {
+    const float a = fabsf(c[i]);
+    if (a == a) mx = max(mx, __float_as_uint(a));
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  unsigned best = 0xffffffffu;
+  for (int i = j + lane_id(); i < n; i += 32)
+    if (__float_as_uint(fabsf(c[i])) == mx) best = min(best, (unsigned)i);
+  best = __reduce_min_sync(0xffffffffu, best);
+  return mx > 0 ? (int)best : -1;
+}
+__device__ __forceinline__ int warp_pivot(int n, int j, const double* c) {
+  double mx = 0;
+  for (int i = j + lane_id(); i < n; i += 32) mx = fmax(mx, fabs(c[i]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  unsigned best = 0xffffffffu;
+  const double band = (1.0 - kPivotTieRtol) * mx;
+  for (int i = j + lane_id(); i < n; i += 32)
+    if (fabs(c[i]) >= band) best = min(best, (unsigned)i);
+  best = __reduce_min_sync(0xffffffffu, best);
+  return mx > 0.0 ? (int)best : -1;
+}
+
+// In-place LU with partial pivoting, P A = L U (unit lower L).  piv[j] = row
+// swapped with j at step j.  Returns false for an exactly zero pivot column.
+// Warp w owns columns w, w + nw, ..: it interchanges and updates them, so a
+// step needs one barrier -- the warp owning column j+1 brings that one up to
+// date first and searches it for the next pivot while the others still work;
+// column j, which everybody reads, is interchanged and scaled in the step
+// after.  (Seven barriers and a float64 reduction per step before: 2 us a step
+// at any size, 560 us for 128 unknowns.)  Every element sees the same operations
+// in the same order as in the plain right-looking form.
 template <typename real>
-__device__ bool cta_lu(int n, real* A, int lda, int* piv, double* red_d, int* red_i,
-                       int* sflag) {
-  (void)sflag;
+__device__ bool cta_lu(int n, real* A, int lda, int* piv, int* spiv) {
   const int lane = lane_id(), warp = warp_id(), nw = num_warps();
+  if (warp == 0) {
+    const int p = warp_pivot(n, 0, A);
+    if (lane == 0) spiv[0] = p;
+  }
+  __syncthreads();
+  int pp = 0;      // the step before: its pivot row and reciprocal
+  real pr = 0;
   for (int j = 0; j < n; j++) {
-    double mx = 0;
-    for (int i = j + threadIdx.x; i < n; i += blockDim.x)
-      mx = fmax(mx, fabs((double)A[i + (int64_t)j * lda]));
-    mx = cta_max_d(mx, red_d);
-    if (!(mx > 0.0)) return false;  // uniform
-    int best = n;
-    for (int i = j + threadIdx.x; i < n; i += blockDim.x)
-      if (fabs((double)A[i + (int64_t)j * lda]) >= (1.0 - kPivotTieRtol) * mx && i < best) best = i;
-    const int p = cta_min_i(best, red_i);
-    if (threadIdx.x == 0) piv[j] = p;
-    if (p != j)
-      for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        real t = A[j + (int64_t)c * lda];
-        A[j + (int64_t)c * lda] = A[p + (int64_t)c * lda];
-        A[p + (int64_t)c * lda] = t;
-      }
-    __syncthreads();
-    // l_ij = a_ij / a_jj is formed on the fly by every column's update and
-    // written back in the next phase
-    const real rd = real(1) / A[j + (int64_t)j * lda];
+    const int p = spiv[j & 1];
+    if (p < 0) return false;  // uniform
     const real* cj = A + (int64_t)j * lda;
-    for (int l = j + 1 + warp; l < n; l += nw) {
+    const real rd = real(1) / cj[p], cjj = cj[j];
+    if (threadIdx.x == 0) piv[j] = p;
+    for (int l = j + 1 + (warp - (j + 1) % nw + nw) % nw; l < n; l += nw) {
       real* cl = A + (int64_t)l * lda;
-      const real ujl = cl[j];
-      for (int i = j + 1 + lane; i < n; i += 32) cl[i] -= (cj[i] * rd) * ujl;
+      const real u = cl[p], down = cl[j];
+      __syncwarp();
+      for (int i = j + 1 + lane; i < n; i += 32) {
+        const real lij = (i == p ? cjj : cj[i]) * rd;
+        cl[i] = (i == p ? down : cl[i]) - lij * u;
+      }
+      if (lane == 0) cl[j] = u;
+      __syncwarp();
+      if (l == j + 1) {
+        const int q = warp_pivot(n, j + 1, cl);
+        if (lane == 0) spiv[(j + 1) & 1] = q;
+      }
     }
-    __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) A[i + (int64_t)j * lda] *= rd;
+    // finish column j - 1, then this step's interchange left of column j
+    if (j > 0 && warp == (j - 1) % nw) {
+      real* c = A + (int64_t)(j - 1) * lda;
+      if (lane == 0 && pp != j - 1) {
+        const real t = c[j - 1];
+        c[j - 1] = c[pp];
+        c[pp] = t;
+      }
+      __syncwarp();
+      for (int i = j + lane; i < n; i += 32) c[i] *= pr;
+      __syncwarp();
+    }
+    if (p != j)
+      for (int c = warp + nw * lane; c < j; c += nw * 32) {
+        real* cc = A + (int64_t)c * lda;
+        const real t = cc[j];
+        cc[j] = cc[p];
+        cc[p] = t;
+      }
+    pp = p;
+    pr = rd;
     __syncthreads();
   }
   return true;
+}
+
+// X = L^{-1} for unit lower triangular L (n x n), out of place, zeros above the
+// diagonal: every column on its own, x_r -= l_ri x_i for i ascending.  A warp
+// keeps four columns in registers (n <= 256), lanes along the rows, and needs no
+// barrier; X must not alias L.
+template <typename real>
+__device__ void cta_trtri_unit(int n, const real* L, int ldl, real* X, int ldx) {
+  constexpr int CW = 4, R = 8;
+  const int lane = lane_id();
+  for (int g0 = warp_id() * CW; g0 < n; g0 += num_warps() * CW) {
+    real x[R][CW];
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int g = 0; g < CW; g++) x[r][g] = lane + 32 * r == g0 + g ? real(1) : real(0);
+#pragma unroll
+    for (int rb = 0; rb < R; rb++) {
+      if (32 * rb + 31 < g0 || 32 * rb >= n) continue;
+      const int hi = min(32, n - 32 * rb);
+      for (int ii = max(0, g0 - 32 * rb); ii < hi; ii++) {
+        const int i = 32 * rb + ii;
+        real xi[CW];
+#pragma unroll
+        for (int g = 0; g < CW; g++) xi[g] = __shfl_sync(0xffffffffu, x[rb][g], ii);
+#pragma unroll
+        for (int r = rb; r < R; r++) {
+          const int row = lane + 32 * r;
+          if (32 * r >= n) break;
+          if (row > i && row < n) {
+            const real l = L[row + (int64_t)i * ldl];
+#pragma unroll
+            for (int g = 0; g < CW; g++) x[r][g] -= l * xi[g];
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int g = 0; g < CW; g++)
+        if (lane + 32 * r < n && g0 + g < n) X[lane + 32 * r + (int64_t)(g0 + g) * ldx] = x[r][g];
+  }
+  __syncthreads();
+}
+
+// V = U^{-1} for upper triangular U (n x n), out of place, zeros below the
+// diagonal: every row on its own, v_il = -(sum over q < l of v_iq u_ql) / u_ll in
+// ascending q.  Four rows per warp, lanes along the columns (n <= 256).
+template <typename real>
+__device__ void cta_trtri_upper_rows(int n, const real* U, int ldu, real* V, int ldv) {
+  constexpr int CW = 4, R = 8;
+  const int lane = lane_id();
+  for (int g0 = warp_id() * CW; g0 < n; g0 += num_warps() * CW) {
+    real acc[R][CW], v[R][CW], d[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int c = lane + 32 * r;
+      d[r] = c < n ? real(1) / U[c + (int64_t)c * ldu] : real(0);
+#pragma unroll
+      for (int g = 0; g < CW; g++) acc[r][g] = v[r][g] = 0;
+    }
+#pragma unroll
+    for (int rb = 0; rb < R; rb++) {
+      if (32 * rb + 31 < g0 || 32 * rb >= n) continue;
+      const int hi = min(32, n - 32 * rb);
+      for (int ll = max(0, g0 - 32 * rb); ll < hi; ll++) {
+        const int l = 32 * rb + ll;
+        real x[CW];
+#pragma unroll
+        for (int g = 0; g < CW; g++) {
+          // this column's entries are final: the lane that holds it
+          const real mine = l == g0 + g ? d[rb] : (l > g0 + g ? -acc[rb][g] * d[rb] : real(0));
+          if (lane == ll) v[rb][g] = mine;
+          x[g] = __shfl_sync(0xffffffffu, mine, ll);
+        }
+#pragma unroll
+        for (int r = rb; r < R; r++) {
+          const int c = lane + 32 * r;
+          if (32 * r >= n) break;
+          if (c > l && c < n) {
+            const real u = U[l + (int64_t)c * ldu];
+#pragma unroll
+            for (int g = 0; g < CW; g++) acc[r][g] += x[g] * u;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++)
+#pragma unroll
+      for (int g = 0; g < CW; g++)
+        if (lane + 32 * r < n && g0 + g < n) V[g0 + g + (int64_t)(lane + 32 * r) * ldv] = v[r][g];
+  }
+  __syncthreads();
 }
 
 // X = L^{-1} for lower triangular L (unit diagonal if `unit`), out of place:
@@ -570,71 +693,71 @@ __device__ void cta_form_q(int m, int k, const real* V, int ldv, const real* tau
 
 // Householder QR without pivoting of the m x k matrix X (column-major, in
 // place): v_j in rows j..m of column j (its head x_jj - beta, beta =
-// -sign(x_jj) ||x_j||), tau[j] = 1 / (r (r + |x_jj|)).  Step j: the warp
-// owning column j forms the reflector; after a barrier every warp applies it
-// to its columns t > j, four at a time (lanes over rows, shuffled dots).
+// -sign(x_jj) ||x_j||), tau[j] = 1 / (r (r + |x_jj|)).  Warp w owns columns
+// w, w + nw, ..; in step j the owner of column j+1 brings it up to date first and
+// forms the next reflector, so a step takes one barrier.
 template <typename real>
 __device__ void cta_qr_np(int m, int k, real* X, int ldx, real* tau) {
-  constexpr int CW = 4;
   const int lane = lane_id(), warp = warp_id(), nw = num_warps();
-  for (int j = 0; j < k; j++) {
-    if (warp == j % nw) {
-      real* xj = X + (int64_t)j * ldx;
-      real sq = 0;
-      for (int i = j + lane; i < m; i += 32) sq += xj[i] * xj[i];
-      sq = warp_sum(sq);
-      const double r = sqrt((double)sq);
-      const double x0 = (double)xj[j];
-      const double beta = (x0 >= 0.0) ? -r : r;
-      const double tj = (r > 0.0) ? 1.0 / (r * (r + fabs(x0))) : 0.0;
-      __syncwarp();
-      if (lane == 0) {
-        xj[j] = (real)(x0 - beta);
-        tau[j] = (real)tj;
-      }
+  const auto form = [&](int j) {  // the owning warp
+    real* xj = X + (int64_t)j * ldx;
+    real sq = 0;
+    for (int i = j + lane; i < m; i += 32) sq += xj[i] * xj[i];
+    sq = warp_sum(sq);
+    const real x0 = xj[j];
+    real head, t;
+    householder_scalars(sq, x0, &head, &t);
+    __syncwarp();
+    if (lane == 0) {
+      xj[j] = head;
+      tau[j] = t;
     }
-    __syncthreads();
+  };
+  if (k > 0 && warp == 0) form(0);
+  __syncthreads();
+  for (int j = 0; j < k; j++) {
     const real* vj = X + (int64_t)j * ldx;
     const real tj = tau[j];
-    for (int t0 = j + 1 + warp; t0 < k; t0 += nw * CW) {
-      real d[CW];
-#pragma unroll
-      for (int g = 0; g < CW; g++) d[g] = 0;
-      for (int i = j + lane; i < m; i += 32) {
-        const real v = vj[i];
-#pragma unroll
-        for (int g = 0; g < CW; g++) {
-          const int t = t0 + g * nw;
-          if (t < k) d[g] += v * X[i + (int64_t)t * ldx];
-        }
-      }
-#pragma unroll
-      for (int g = 0; g < CW; g++) d[g] = warp_sum(d[g]) * tj;
-      for (int i = j + lane; i < m; i += 32) {
-        const real v = vj[i];
-#pragma unroll
-        for (int g = 0; g < CW; g++) {
-          const int t = t0 + g * nw;
-          if (t < k) X[i + (int64_t)t * ldx] -= d[g] * v;
-        }
-      }
+    for (int t = j + 1 + (warp - (j + 1) % nw + nw) % nw; t < k; t += nw) {
+      real* xt = X + (int64_t)t * ldx;
+      real d = 0;
+      for (int i = j + lane; i < m; i += 32) d += vj[i] * xt[i];
+      d = warp_sum(d) * tj;
+      for (int i = j + lane; i < m; i += 32) xt[i] -= d * vj[i];
+      __syncwarp();
+      if (t == j + 1) form(t);
     }
     __syncthreads();
   }
 }
 
-// Column permutation of the LU inverse: (X P)[:, c] = X[:, pos(c)], pos(c) =
-// row of P A holding original row c after the swaps piv[0..n-1] in order.
-template <typename real>
-__device__ void cta_permute_cols(int n, const int* piv, const real* X, int ldx, real* Y, int ldy) {
+// pos[c] = row of P A holding original row c after the swaps piv[0..n-1] in
+// order (inverse = false), or the original row that row c of P A holds.
+__device__ void cta_permutation(int n, const int* piv, int* pos, bool inverse) {
   for (int c = threadIdx.x; c < n; c += blockDim.x) {
-    int pos = c;
-    for (int j = 0; j < n; j++) {
-      if (piv[j] == pos) pos = j;
-      else if (j == pos) pos = piv[j];
+    int q = c;
+    if (!inverse) {
+      for (int j = 0; j < n; j++) {
+        const int p = piv[j];
+        q = p == q ? j : (j == q ? p : q);
+      }
+    } else {
+      for (int j = n - 1; j >= 0; j--) {
+        const int p = piv[j];
+        q = p == q ? j : (j == q ? p : q);
+      }
     }
-    for (int i = 0; i < n; i++) Y[i + (int64_t)c * ldy] = X[i + (int64_t)pos * ldx];
+    pos[c] = q;
   }
+  __syncthreads();
+}
+
+// Y = X P: column c of Y is column pos[c] of X.
+template <typename real>
+__device__ void cta_permute_cols(int n, const int* pos, const real* X, int ldx, real* Y, int ldy) {
+  for (int c = warp_id(); c < n; c += num_warps())
+    for (int i = lane_id(); i < n; i += 32)
+      Y[i + (int64_t)c * ldy] = X[i + (int64_t)pos[c] * ldx];
   __syncthreads();
 }
 
@@ -662,7 +785,6 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
   __shared__ int sflag;
   __shared__ int s_ncol;
   __shared__ double s_amax;
-  __shared__ real gsh[2 * GK * (GT + 1)];
   extern __shared__ unsigned char dsm[];
   const PrepTask tk = tasks[blockIdx.x];
   const int m = tk.m;
@@ -704,20 +826,21 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
   real* tau2 = tau + m;
   real* rsign = tau2 + m;  // sign of R's diagonal in the pivoted QR
   int* piv = reinterpret_cast<int*>(rsign + m);
+  int* pos = reinterpret_cast<int*>(vsh);  // m ints (vsh: the in-kernel QR's, spent by then)
   real* T = fac + tk.T;
 
   // ---- A_ss, its largest magnitude (scale of the noise floor), its factor
   cta_copy<real>(m, m, arena + tk.a_ss, tk.ld, W_A, ldA);
   {
-    double mx = 0;
-    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x)
-      mx = fmax(mx, fabs((double)W_A[idx % m + (int64_t)(idx / m) * ldA]));
-    mx = cta_max_d(mx, red_d);
-    if (threadIdx.x == 0) s_amax = mx;
+    real mx = 0;  // (the float64 pipe issues two lanes per clock)
+    for (int j = warp_id(); j < m; j += num_warps())
+      for (int i = lane_id(); i < m; i += 32) mx = fmax(mx, fabs(W_A[i + (int64_t)j * ldA]));
+    const double all = cta_max_d((double)mx, red_d);
+    if (threadIdx.x == 0) s_amax = all;
     __syncthreads();
   }
   const bool ok = sym ? cta_cholesky<real>(m, W_A, ldA, &sflag)
-                      : cta_lu<real>(m, W_A, ldA, piv, red_d, red_i, &sflag);
+                      : cta_lu<real>(m, W_A, ldA, piv, red_i);
   if (!ok) {
     report<real>(err, sym ? (int)HSOLVE_ERR_NOT_SPD : (int)HSOLVE_ERR_SINGULAR, tk.s, level, rank, m);
     return;
@@ -835,7 +958,7 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
       cta_copy<real>(m, m, W_B, ldB, T, m);
       return;
     }
-    cta_gemm<real>(m, m, m, W_B, ldB, true, W_B, ldB, false, W_A, ldA, real(1), real(0), gsh);
+    cta_gemm<real>(m, m, m, W_B, ldB, true, W_B, ldB, false, W_A, ldA);
     real* tp = W_A;
     W_A = W_B;
     W_B = tp;
@@ -844,13 +967,19 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
     ldB = tl;
   } else {
     // L^{-1} (unit lower) into W_L, U^{-1} into W_S
-    cta_trtri_lower_oop<real>(m, W_A, ldA, true, W_L, m);
-    cta_copy<real>(m, m, W_A, ldA, W_S, m);
-    cta_trtri_upper<real>(m, W_S, m, tsh);
-    cta_zero_tri<real>(m, W_S, m, false);
+    if (m <= kRowsMax) {
+      cta_trtri_unit<real>(m, W_A, ldA, W_L, m);
+      cta_trtri_upper_rows<real>(m, W_A, ldA, W_S, m);
+    } else {
+      cta_trtri_lower_oop<real>(m, W_A, ldA, true, W_L, m);
+      cta_copy<real>(m, m, W_A, ldA, W_S, m);
+      cta_trtri_upper<real>(m, W_S, m, tsh);
+      cta_zero_tri<real>(m, W_S, m, false);
+    }
+    cta_permutation(m, piv, pos, false);
     if (k == 0) {
       // E_s = I: T' = L^{-1} P, T'_R^T = (U^{-1})^T
-      cta_permute_cols<real>(m, piv, W_L, m, T, m);
+      cta_permute_cols<real>(m, pos, W_L, m, T, m);
       real* TRt = fac + tk.TR;
       for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
         int i = idx % m, j = idx / m;
@@ -860,8 +989,8 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
       return;
     }
     // B = U^{-1} L^{-1} P
-    cta_gemm<real>(m, m, m, W_S, m, false, W_L, m, false, W_F, m, real(1), real(0), gsh);
-    cta_permute_cols<real>(m, piv, W_F, m, W_B, ldB);
+    cta_gemm<real>(m, m, m, W_S, m, false, W_L, m, false, W_F, m);
+    cta_permute_cols<real>(m, pos, W_F, m, W_B, ldB);
   }
 
   mark(4);
@@ -877,22 +1006,19 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
   }
   __syncthreads();
 
-  // ---- V_L: complement of X = B U (full QR of X, V = Q[:, k:]); in the SPD
-  // case X takes the (spent) shared-memory home of the factor of A_ss
-  int ldX = m;
-  if (sym) {
-    W_X = W_A;
-    ldX = ldA;
-  }
-  cta_gemm<real>(m, k, m, W_B, ldB, false, W_U, ldU, false, W_X, ldX, real(1), real(0), gsh);
+  // ---- V_L: complement of X = B U (full QR of X, V = Q[:, k:]); X takes the
+  // (spent) home of the factor of A_ss
+  W_X = W_A;
+  const int ldX = ldA;
+  cta_gemm<real>(m, k, m, W_B, ldB, false, W_U, ldU, false, W_X, ldX);
   cta_qr_np<real>(m, k, W_X, ldX, tau2);
   W_V = W_U + (int64_t)k * ldU;
   cta_form_q<real, false>(m, k, W_X, ldX, tau2, k, f, W_V, ldU, vsh);
 
   mark(5);
   // ---- T = [U V_L]^T B (one product); C = U^T B U -> coarse (s,s) block
-  cta_gemm<real>(m, m, m, W_U, ldU, true, W_B, ldB, false, W_T, m, real(1), real(0), gsh);
-  cta_gemm<real>(k, k, m, W_T, m, false, W_U, ldU, false, W_C, m, real(1), real(0), gsh);
+  cta_gemm<real>(m, m, m, W_U, ldU, true, W_B, ldB, false, W_T, m);
+  cta_gemm<real>(k, k, m, W_T, m, false, W_U, ldU, false, W_C, m);
 
   if (sym) {
     // F = V^T B V; L_F^{-1}; T' rows k.. = L_F^{-1} V^T B.  F lives where the
@@ -900,53 +1026,57 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
     W_F = W_A;
     const int ldF = ldA;
     mark(6);
-    cta_gemm<real>(f, f, m, W_T + k, m, false, W_V, ldU, false, W_F, ldF, real(1), real(0), gsh);
+    cta_gemm<real>(f, f, m, W_T + k, m, false, W_V, ldU, false, W_F, ldF);
     if (!cta_cholesky<real>(f, W_F, ldF, &sflag)) {
       report<real>(err, (int)HSOLVE_ERR_NOT_SPD, tk.s, level, rank, m);
       return;
     }
     cta_trtri_lower_oop<real>(f, W_F, ldF, false, W_L, m);
     cta_copy<real>(k, m, W_T, m, T, m);
-    cta_gemm<real>(f, m, f, W_L, m, false, W_T + k, m, false, T + k, m, real(1), real(0), gsh);
+    cta_gemm<real>(f, m, f, W_L, m, false, W_T + k, m, false, T + k, m);
     // D = C U^T (k x m) for the coarse-to-far update C (U^T A_sw)
-    cta_gemm<real>(k, m, k, W_C, m, false, W_U, ldU, true, ws_all + tk.D, m, real(1), real(0),
-                   gsh);
+    cta_gemm<real>(k, m, k, W_C, m, false, W_U, ldU, true, ws_all + tk.D, m);
   } else {
     // V_R: complement of B^T U
-    cta_gemm<real>(m, k, m, W_B, ldB, true, W_U, ldU, false, W_X, m, real(1), real(0), gsh);
-    cta_qr_np<real>(m, k, W_X, m, tau2);
-    cta_form_q<real, false>(m, k, W_X, m, tau2, k, f, W_R, m, vsh);
-    // F = V_L^T B V_R (f x f) and its LU
-    cta_gemm<real>(f, f, m, W_T + k, m, false, W_R, m, false, W_F, m, real(1), real(0), gsh);
-    if (!cta_lu<real>(f, W_F, m, piv, red_d, red_i, &sflag)) {
+    cta_gemm<real>(m, k, m, W_B, ldB, true, W_U, ldU, false, W_X, ldX);
+    cta_qr_np<real>(m, k, W_X, ldX, tau2);
+    cta_form_q<real, false>(m, k, W_X, ldX, tau2, k, f, W_R, m, vsh);
+    // F = V_L^T B V_R (f x f) and its LU, in the home of X
+    W_F = W_A;
+    const int ldF = ldA;
+    cta_gemm<real>(f, f, m, W_T + k, m, false, W_R, m, false, W_F, ldF);
+    if (!cta_lu<real>(f, W_F, ldF, piv, red_i)) {
       report<real>(err, (int)HSOLVE_ERR_SINGULAR, tk.s, level, rank, m);
       return;
     }
-    // T' rows k.. = L_F^{-1} P_F V_L^T B: permute rows of W_T[k:] by piv
-    for (int j = 0; j < f; j++) {
-      const int p = piv[j];
-      if (p != j)
-        for (int c = threadIdx.x; c < m; c += blockDim.x) {
-          real t = W_T[k + j + (int64_t)c * m];
-          W_T[k + j + (int64_t)c * m] = W_T[k + p + (int64_t)c * m];
-          W_T[k + p + (int64_t)c * m] = t;
-        }
-      __syncthreads();
-    }
-    cta_trtri_lower_oop<real>(f, W_F, m, true, W_L, m);
+    // T' rows k.. = L_F^{-1} P_F V_L^T B; P_F V_L^T B beside the workspace's
+    // spent inverse, L_F^{-1} over the spent V_L
+    cta_permutation(f, piv, pos, true);
+    real* W_P = ws + 5 * mm;
+    for (int c = warp_id(); c < m; c += num_warps())
+      for (int i = lane_id(); i < f; i += 32)
+        W_P[i + (int64_t)c * m] = W_T[k + pos[i] + (int64_t)c * m];
+    if (f <= kRowsMax) cta_trtri_unit<real>(f, W_F, ldF, W_L, m);
+    else cta_trtri_lower_oop<real>(f, W_F, ldF, true, W_L, m);
     cta_copy<real>(k, m, W_T, m, T, m);
-    cta_gemm<real>(f, m, f, W_L, m, false, W_T + k, m, false, T + k, m, real(1), real(0), gsh);
+    cta_gemm<real>(f, m, f, W_L, m, false, W_P, m, false, T + k, m);
     // T'_R = B [U, V_R U_F^{-1}]; store its transpose
-    cta_trtri_upper<real>(f, W_F, m, tsh);
-    cta_zero_tri<real>(f, W_F, m, false);
-    cta_gemm<real>(m, f, f, W_R, m, false, W_F, m, false, W_S, m, real(1), real(0), gsh);
+    const real* W_Ui = W_F;
+    int ldi = ldF;
+    if (f <= kRowsMax) {
+      cta_trtri_upper_rows<real>(f, W_F, ldF, W_L, m);
+      W_Ui = W_L;
+      ldi = m;
+    } else {
+      cta_trtri_upper<real>(f, W_F, ldF, tsh);
+      cta_zero_tri<real>(f, W_F, ldF, false);
+    }
+    cta_gemm<real>(m, f, f, W_R, m, false, W_Ui, ldi, false, W_S, m);
     real* TRt = fac + tk.TR;
-    cta_gemm<real>(k, m, m, W_U, ldU, true, W_B, ldB, true, TRt, m, real(1), real(0), gsh);
-    cta_gemm<real>(f, m, m, W_S, m, true, W_B, ldB, true, TRt + k, m, real(1), real(0), gsh);
-    cta_gemm<real>(k, m, k, W_C, m, false, W_U, ldU, true, ws_all + tk.D, m, real(1), real(0),
-                   gsh);
-    cta_gemm<real>(k, m, k, W_C, m, true, W_U, ldU, true, ws_all + tk.D2, m, real(1), real(0),
-                   gsh);
+    cta_gemm<real>(k, m, m, W_U, ldU, true, W_B, ldB, true, TRt, m);
+    cta_gemm<real>(f, m, m, W_S, m, true, W_B, ldB, true, TRt + k, m);
+    cta_gemm<real>(k, m, k, W_C, m, false, W_U, ldU, true, ws_all + tk.D, m);
+    cta_gemm<real>(k, m, k, W_C, m, true, W_U, ldU, true, ws_all + tk.D2, m);
   }
   // write C into the (s,s) block (coarse part); done last: A_ss was copied
   real* blk_ss = arena + tk.a_ss;
@@ -970,7 +1100,7 @@ void Launch<real>::prep(const PrepTask* tasks_dev, int ntask, real* arena, real*
   // oracle's 1e-14 in float64; float32 blocks carry ~1e-7 relative noise
   const double noise_rtol = sizeof(real) == 8 ? 1e-14 : 1e-6;
   // the factor of A_ss and A_ss^{-1} in shared memory when they fit
-  const size_t budget = 220 * 1024 - 2 * GK * (GT + 1) * sizeof(real) - 4 * 1024;
+  const size_t budget = 208 * 1024;
   const size_t one = sizeof(real) * (size_t)(maxm | 1) * maxm;
   const size_t vec = sizeof(real) * 2 * (size_t)maxm;
   int mats = 0;
