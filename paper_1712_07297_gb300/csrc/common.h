@@ -237,8 +237,12 @@ void mbar_wait_probe(long long limit, int* err, cudaStream_t st);
 void tc_gemm(int mode, int M, int N, int K, const float* A, int64_t rsa, int64_t csa,
              const float* B, int64_t rsb, int64_t csb, float* C, int64_t ldc, float alpha,
              float beta, bool lower, DevError* err, cudaStream_t st);
-// Dense top on tensor cores (float32, SPD): L into A's lower triangle, X =
-// L^{-1} (ld n); W: dense_top_tc_scratch(n) floats.
+// X = L^{-1} for the Cholesky factor L of the lower n x n block at A (n <= 128),
+// one CTA (kernels_spd.cu).
+void chol_inv_leaf(float* A, int64_t lda, float* X, int64_t ldx, int n, DevError* err, int level,
+                   cudaStream_t st);
+// Dense top on tensor cores (float32, SPD): X = L^{-1} (ld n), A's lower triangle
+// is used up; W: dense_top_tc_scratch(n) floats.
 size_t dense_top_tc_scratch(int n);
 // Schur-complement update of a colour class (the SIMT schur launch's
 // arguments) with tensor-core products in the given mode.

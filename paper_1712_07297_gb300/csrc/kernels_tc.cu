@@ -16,7 +16,7 @@
 // tensor memory.
 //
 // The dense top (SPD, float32) uses the recursive blocked form
-//   L11 = chol(A11), X11 = L11^{-1}   (recursively; 128-wide leaves on one CTA)
+//   X11 = chol(A11)^{-1}   (recursively; 128-wide leaves on one CTA)
 //   L21 = A21 X11^T,  A22 -= L21 L21^T,  L22 = chol(A22), X22 = L22^{-1}
 //   X21 = -X22 (L21 X11)
 // so that all but the leaves are tensor-core products.
@@ -502,139 +502,7 @@ schur_tc_kernel(const SchurTask* __restrict__ tasks, const float* __restrict__ f
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TN));
 }
 
-// ---- dense top leaves: Cholesky and inverse factor of an n <= 128 block on
-// one CTA (lower triangle of A in, L into A's lower triangle, X = L^{-1}
-// into X with zeros above the diagonal)
-constexpr int kLeaf = 128;
-
-// 256 threads as a 16 x 16 grid; thread (tr, tc) keeps the elements (tr +
-// 16 a, tc + 16 b), a, b < 8, of the factor (and then of the inverse) in
-// registers, so a step reads 16 broadcast values from shared memory and
-// updates up to 64 registers; two barriers per step.  The pivots come from a
-// shared copy of the trailing diagonal updated alongside.
-__global__ void __launch_bounds__(256, 1)
-chol_inv_leaf_kernel(float* A, int64_t lda, float* X, int64_t ldx, int n, DevError* err,
-                     int level) {
-  constexpr int G = 16, R8 = kLeaf / G;
-  extern __shared__ float leaf_smem[];
-  const int ld = kLeaf + 1;
-  float* Ls = leaf_smem;                // L, column-major (for the inverse)
-  float* vec = leaf_smem + ld * kLeaf;  // the step's column / row
-  __shared__ float diag[kLeaf];         // the trailing diagonal (the pivots)
-  const int tr = threadIdx.x % G, tc = threadIdx.x / G;
-  float R[R8][R8];
-#pragma unroll
-  for (int a = 0; a < R8; a++)
-#pragma unroll
-    for (int b = 0; b < R8; b++) {
-      const int i = tr + G * a, l = tc + G * b;
-      R[a][b] = (i < n && l < n && i >= l) ? A[i + (int64_t)l * lda] : 0.f;
-    }
-  for (int t = threadIdx.x; t < n; t += blockDim.x) diag[t] = A[t + (int64_t)t * lda];
-  __syncthreads();
-  // ---- Cholesky, right-looking: scale column j, then update the trailing part
-  for (int j = 0; j < n; j++) {
-    const float d = diag[j];
-    if (!(d > 0.f)) {
-      if (threadIdx.x == 0 && atomicCAS(&err->code, 0, (int)HSOLVE_ERR_NOT_SPD) == 0) {
-        err->cluster = 0;
-        err->level = level;
-      }
-      return;  // uniform
-    }
-    const float rs = rsqrtf(d);
-    const int jb = j / G;
-    if (tc == j % G) {
-#pragma unroll
-      for (int a = 0; a < R8; a++) {
-        const int i = tr + G * a;
-#pragma unroll
-        for (int b = 0; b < R8; b++)
-          if (b == jb && i >= j && i < n) {
-            R[a][b] = (i == j) ? d * rs : R[a][b] * rs;
-            vec[i] = R[a][b];
-          }
-      }
-    }
-    __syncthreads();
-    float ci[R8], cl[R8];
-#pragma unroll
-    for (int a = 0; a < R8; a++) {
-      const int i = tr + G * a;
-      ci[a] = (i > j && i < n) ? vec[i] : 0.f;
-    }
-#pragma unroll
-    for (int b = 0; b < R8; b++) {
-      const int l = tc + G * b;
-      cl[b] = (l > j && l < n) ? vec[l] : 0.f;
-    }
-#pragma unroll
-    for (int a = 0; a < R8; a++)
-#pragma unroll
-      for (int b = 0; b < R8; b++) {
-        const int i = tr + G * a, l = tc + G * b;
-        if (i >= l) R[a][b] -= ci[a] * cl[b];
-      }
-    // the pivots of the later steps
-    for (int t = j + 1 + threadIdx.x; t < n; t += blockDim.x) diag[t] -= vec[t] * vec[t];
-    __syncthreads();
-  }
-  // ---- L to shared memory and global; R becomes Y = L^{-1}, from I
-#pragma unroll
-  for (int a = 0; a < R8; a++)
-#pragma unroll
-    for (int b = 0; b < R8; b++) {
-      const int i = tr + G * a, l = tc + G * b;
-      if (i < n && l < n) {
-        Ls[i + l * ld] = (i >= l) ? R[a][b] : 0.f;
-        if (i >= l) A[i + (int64_t)l * lda] = R[a][b];
-      }
-      R[a][b] = (i == l && i < n) ? 1.f : 0.f;
-    }
-  __syncthreads();
-  // forward substitution on all columns at once: step i scales row i by
-  // 1 / l_ii, then y_rc -= l_ri y_ic for r > i, c <= i
-  for (int i = 0; i < n; i++) {
-    const float di = 1.f / Ls[i + i * ld];
-    const int ib = i / G;
-    if (tr == i % G) {
-#pragma unroll
-      for (int a = 0; a < R8; a++)
-#pragma unroll
-        for (int b = 0; b < R8; b++) {
-          const int c = tc + G * b;
-          if (a == ib && c <= i) {
-            R[a][b] *= di;
-            vec[c] = R[a][b];
-          }
-        }
-    }
-    __syncthreads();
-    float lr[R8], yc[R8];
-#pragma unroll
-    for (int a = 0; a < R8; a++) {
-      const int r = tr + G * a;
-      lr[a] = (r > i && r < n) ? Ls[r + i * ld] : 0.f;
-    }
-#pragma unroll
-    for (int b = 0; b < R8; b++) {
-      const int c = tc + G * b;
-      yc[b] = (c <= i) ? vec[c] : 0.f;
-    }
-#pragma unroll
-    for (int a = 0; a < R8; a++)
-#pragma unroll
-      for (int b = 0; b < R8; b++) R[a][b] -= lr[a] * yc[b];
-    __syncthreads();
-  }
-#pragma unroll
-  for (int a = 0; a < R8; a++)
-#pragma unroll
-    for (int b = 0; b < R8; b++) {
-      const int i = tr + G * a, c = tc + G * b;
-      if (i < n && c < n) X[i + (int64_t)c * ldx] = (i >= c) ? R[a][b] : 0.f;
-    }
-}
+constexpr int kLeaf = 128;  // dense top leaves: chol_inv_leaf (kernels_spd.cu)
 
 __global__ void copy_block_kernel(const float* __restrict__ src, int64_t lds, float* dst,
                                   int64_t ldd, int rows, int cols) {
@@ -673,20 +541,12 @@ void launch_gemm(int M, int N, int K, const float* A, int64_t rsa, int64_t csa, 
 
 int grid1(int64_t work) { return (int)std::min<int64_t>((work + 255) / 256, 152 * 8); }
 
-// Recursive Cholesky + inverse factor of the n x n SPD block at A (lower part),
-// X = L^{-1} (ld ldx).  W: scratch of at least n * n / 4 floats.
+// Recursive Cholesky + inverse factor of the n x n SPD block at A (lower part,
+// used up: off its diagonal blocks of 128 it ends as L), X = L^{-1} (ld ldx).  W: scratch of at least n * n / 4 floats.
 void top_rec(float* A, int64_t lda, float* X, int64_t ldx, int n, float* W, DevError* err,
              int level, cudaStream_t st) {
   if (n <= kLeaf) {
-    const size_t smem = ((size_t)(kLeaf + 1) * kLeaf + kLeaf) * sizeof(float);
-    static const bool attr_set = [smem] {
-      cudaFuncSetAttribute(chol_inv_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      return true;
-    }();
-    (void)attr_set;
-    count_launch();
-    chol_inv_leaf_kernel<<<1, 256, smem, st>>>(A, lda, X, ldx, n, err, level);
+    chol_inv_leaf(A, lda, X, ldx, n, err, level, st);
     return;
   }
   // split at a multiple of the leaf size near the middle
