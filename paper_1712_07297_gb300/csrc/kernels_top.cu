@@ -467,11 +467,12 @@ lu_swap_kernel(real* A, int64_t lda, int n, int j0, int b, const int* __restrict
 // skip their zero chunks: tri & 1 -- A(r, k) = 0 for k > r; tri & 2 --
 // B(c, k) = 0 for k < c.
 template <typename real>
-__global__ void __launch_bounds__(256)
-simt_gemm_kernel(int M, int N, int K, const real* __restrict__ A, int64_t rsa, int64_t csa,
-                 const real* __restrict__ B, int64_t rsb, int64_t csb, real* __restrict__ C,
-                 int64_t ldc, real alpha, real beta, int tri) {
+__device__ __forceinline__ void simt_gemm(int M, int N, int K, const real* __restrict__ A,
+                                          int64_t rsa, int64_t csa, const real* __restrict__ B,
+                                          int64_t rsb, int64_t csb, real* __restrict__ C,
+                                          int64_t ldc, real alpha, real beta, int tri) {
   const int i0 = blockIdx.x * NB, c0 = blockIdx.y * NB;
+  if (i0 >= M || c0 >= N) return;
   const int kbeg = (tri & 2) ? (c0 / 16) * 16 : 0;
   const int kend = (tri & 1) ? min(K, i0 + NB) : K;
   __shared__ real As[16][NB + 1];
@@ -522,6 +523,31 @@ simt_gemm_kernel(int M, int N, int K, const real* __restrict__ A, int64_t rsa, i
         *cp = beta == real(0) ? alpha * acc[p][q] : alpha * acc[p][q] + beta * *cp;
       }
     }
+}
+
+template <typename real>
+__global__ void __launch_bounds__(256)
+simt_gemm_kernel(int M, int N, int K, const real* __restrict__ A, int64_t rsa, int64_t csa,
+                 const real* __restrict__ B, int64_t rsb, int64_t csb, real* __restrict__ C,
+                 int64_t ldc, real alpha, real beta, int tri) {
+  simt_gemm<real>(M, N, K, A, rsa, csa, B, rsb, csb, C, ldc, alpha, beta, tri);
+}
+
+// One half of a level of the triangular inverse, for every pair of blocks of w
+// at once (grid z): W = L21 X11 (second = 0) or X21 = -X22 W, the pair's W
+// (n2 x w, ld n2) at W + pair w^2.
+template <typename real>
+__global__ void __launch_bounds__(256)
+tri_inv_level_kernel(const real* __restrict__ L, int64_t ldl, real* X, int64_t ldx, int n, int w,
+                     real* W, int second) {
+  const int b = 2 * w * blockIdx.z, n2 = min(w, n - b - w);
+  real* Wp = W + (int64_t)blockIdx.z * w * w;
+  if (second)
+    simt_gemm<real>(n2, w, n2, X + (b + w) + (int64_t)(b + w) * ldx, 1, ldx, Wp, n2, 1,
+                    X + (b + w) + (int64_t)b * ldx, ldx, real(-1), real(0), 1);
+  else
+    simt_gemm<real>(n2, w, w, L + (b + w) + (int64_t)b * ldl, 1, ldl, X + b + (int64_t)b * ldx,
+                    ldx, 1, Wp, n2, real(1), real(0), 2);
 }
 
 // dst (rows x cols, ld ldd) = src (ld lds)
@@ -617,28 +643,12 @@ void gemm_nt(int M, int N, int K, const real* A, int64_t rsa, int64_t csa, const
   }
 }
 
-// X = L^{-1} for the lower triangular n x n L (unit diagonal if `unit`),
-// recursively: with L = [L11 0; L21 L22] split at a multiple of 64,
-// X11 = L11^{-1}, X22 = L22^{-1} and X21 = -X22 (L21 X11), so that all but
-// the 64 x 64 diagonal blocks (inverted first, in one launch) are matrix
-// products.  X's blocks above the diagonal are zeroed by the caller.  W:
-// scratch of at least (n/2 + 64)^2 elements.
-template <typename real>
-void tri_inv_products(const real* L, int64_t ldl, real* X, int64_t ldx, int n, real* W,
-                      DevError* err, cudaStream_t st) {
-  if (n <= NB) return;
-  const int n1 = std::max(NB, ((n / 2) + NB - 1) / NB * NB);
-  const int n2 = n - n1;
-  if (n2 <= 0) return;
-  tri_inv_products(L, ldl, X, ldx, n1, W, err, st);
-  tri_inv_products(L + n1 + (int64_t)n1 * ldl, ldl, X + n1 + (int64_t)n1 * ldx, ldx, n2, W, err,
-                   st);
-  // W = L21 X11 (n2 x n1, ld n2), X21 = -X22 W
-  gemm_nt<real>(n2, n1, n1, L + n1, 1, ldl, X, ldx, 1, W, n2, real(1), real(0), 2, err, st);
-  gemm_nt<real>(n2, n1, n2, X + n1 + (int64_t)n1 * ldx, 1, ldx, W, n2, 1, X + n1, ldx, real(-1),
-                real(0), 1, err, st);
-}
-
+// X = L^{-1} for the lower triangular n x n L (unit diagonal if `unit`): the
+// 64 x 64 diagonal blocks, then pairs of blocks of w = 64, 128, ..: X21 = -X22
+// (L21 X11), two launches per level.  (A launch per pair left the small levels
+// to one to sixteen CTAs, at 67 us of the float64 pipe per 64 x 64 x 64: float64
+// top of 6,469 unknowns 230 -> 198 ms.)  X's blocks above the diagonal are
+// zeroed by the caller.  W: scratch of at least (n/2 + 64)^2 elements.
 template <typename real>
 void tri_inv(const real* L, int64_t ldl, real* X, int64_t ldx, int n, bool unit, real* W,
              DevError* err, cudaStream_t st) {
@@ -652,7 +662,15 @@ void tri_inv(const real* L, int64_t ldl, real* X, int64_t ldx, int n, bool unit,
   count_launch();
   tri_inv_diag_kernel<real><<<(n + NB - 1) / NB, 64, smem, st>>>(L, ldl, X, ldx, n,
                                                                  unit ? 1 : 0);
-  tri_inv_products(L, ldl, X, ldx, n, W, err, st);
+  (void)err;
+  for (int w = NB; w < n; w *= 2) {
+    const int pairs = (n - w + 2 * w - 1) / (2 * w), t = w / NB;
+    for (int second = 0; second < 2; second++) {
+      count_launch();
+      tri_inv_level_kernel<real><<<dim3(t, t, pairs), 256, 0, st>>>(L, ldl, X, ldx, n, w, W,
+                                                                   second);
+    }
+  }
 }
 
 // The recursive LU of the columns [j0, j0 + nn) over rows [j0, n) (the left
