@@ -224,6 +224,7 @@ struct hsolve_handle {
   DevBuf top_w;  // scratch of the tensor-core dense top
   PinnedBuf pin, pin2, pin3;
   PinnedBuf pin_rank;  // ranks and error words copied back class by class
+  PinnedBuf pin_cnt;   // nonzero fill columns of a class
   // CUDA graphs of the substitution sweeps, one per nrhs (dropped whenever
   // the factorization or the level buffers change)
   bool use_graphs = true;
@@ -1129,17 +1130,25 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
         Launch<real>::count_nz(d_qrt, (int)qrt.size(), qc, arena, h->wsd.as<double>(), d_segs,
                                h->cnt.as<int>(), h->st);
       });
-      std::vector<int> cnt(qrt.size());
+      h->pin_cnt.ensure(sizeof(int) * qrt.size());
+      const int* pcnt = reinterpret_cast<const int*>(h->pin_cnt.p);
       {
         HostTimer ht(h, "host.count_copy");
-        HS_CUDA(cudaMemcpyAsync(cnt.data(), h->cnt.p, sizeof(int) * cnt.size(),
+        HS_CUDA(cudaMemcpyAsync(h->pin_cnt.p, h->cnt.p, sizeof(int) * qrt.size(),
                                 cudaMemcpyDeviceToHost, h->st));
       }
-      {
+      // A class whose gathered columns, zero ones included, fit the register
+      // form on the chip at once needs no count before its launch; the others
+      // wait for it (25 us of an idle device per class).
+      int early_CL = 0;
+      const int early = sym ? Launch<real>::qr_reg_form(qm, qc, &early_CL) : -1;
+      const bool counted = !(early >= 0 && (int64_t)qrt.size() * early_CL <= kNumSMs);
+      if (counted) {
         HostTimer ht(h, "host.wait_count");
         HS_CUDA(cudaStreamSynchronize(h->st));
       }
-      for (size_t i = 0; i < qrt.size(); i++) nzcols[qrt[i].s] = cnt[i];
+      std::vector<int> cnt(qrt.size());
+      for (size_t i = 0; i < qrt.size(); i++) cnt[i] = counted ? pcnt[i] : qrt[i].ncolG;
       // The float32 SPD path keeps columns in registers (form, CTAs per
       // cluster).  A class that fits the chip at once takes the form of its
       // largest task; in a larger one every task takes the form its own size
@@ -1293,6 +1302,9 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
       HS_CUDA(cudaEventSynchronize(ev_rank));
     }
     if (nclass > 0) check_err_copy(kerr[(nclass - 1) & 1]);
+    // (copied before the ranks)
+    for (size_t i = 0; i < qrt.size(); i++)
+      nzcols[qrt[i].s] = reinterpret_cast<const int*>(h->pin_cnt.p)[i];
     std::vector<int> kk(krank, krank + nc);
     for (int s : S) {
       FL.k[s] = kk[s];
