@@ -525,50 +525,80 @@ __device__ __forceinline__ void group_reduce(real* a, int lane, int* base) {
   }
 }
 
-// out(o, r) = sum_l A[o * lda + l] v[l][r] for o < nout: eight lanes share an
-// output, 32 outputs per pass of the CTA.  emit(o, r, value) is called once
+// out(o, r) = sum_l A[o * lda + l] v[l][r] for o < nout: eight lanes share NO
+// outputs, 32 NO outputs per pass of the CTA.  emit(o, r, value) is called once
 // per output and right-hand side.
-template <typename real, int RB, typename Emit>
-__device__ __forceinline__ void sweep_dots(const real* A, int lda, int nout, int inner,
-                                           const real* v, Emit&& emit) {
+template <typename real, int RB, int NO, typename Emit>
+__device__ __forceinline__ void sweep_dots_by(const real* A, int lda, int nout, int inner,
+                                              const real* v, Emit& emit) {
   constexpr int VS = VecStride<real, RB>::value;
   constexpr int kLeft = RB >= 8 ? RB / 8 : 1;  // values a lane ends with
-  const int lane = threadIdx.x & 31, p = threadIdx.x & 7;
-  for (int o0 = threadIdx.x >> 3; o0 - (int)(threadIdx.x >> 3) < nout; o0 += kSweepThreads / 8) {
-    const int o = min(o0, nout - 1);
-    const real* row = A + o * lda;
-    real acc[RB];
+  constexpr int kGroups = kSweepThreads / 8;
+  const int lane = threadIdx.x & 31, p = threadIdx.x & 7, g = threadIdx.x >> 3;
+  for (int base0 = 0; base0 < nout; base0 += kGroups * NO) {
+    const real* row[NO];
 #pragma unroll
-    for (int r = 0; r < RB; r++) acc[r] = 0;
+    for (int w = 0; w < NO; w++) row[w] = A + min(base0 + g + w * kGroups, nout - 1) * lda;
+    real acc[NO][RB];
+#pragma unroll
+    for (int w = 0; w < NO; w++)
+#pragma unroll
+      for (int r = 0; r < RB; r++) acc[w][r] = 0;
+    constexpr int kUnroll = NO * RB >= 32 ? 1 : (NO * RB >= 8 ? 2 : 4);
     int l = p;
-    constexpr int kUnroll = RB >= 32 ? 1 : (RB >= 8 ? 2 : 4);
     for (; l + 8 * (kUnroll - 1) < inner; l += 8 * kUnroll) {
-      real a[kUnroll];
+      real a[kUnroll][NO];
 #pragma unroll
-      for (int u = 0; u < kUnroll; u++) a[u] = row[l + 8 * u];
+      for (int u = 0; u < kUnroll; u++)
+#pragma unroll
+        for (int w = 0; w < NO; w++) a[u][w] = row[w][l + 8 * u];
 #pragma unroll
       for (int u = 0; u < kUnroll; u++) {
         real x[RB];
         load_vec<real, RB>(v + (l + 8 * u) * VS, x);
 #pragma unroll
-        for (int r = 0; r < RB; r++) acc[r] += a[u] * x[r];
+        for (int w = 0; w < NO; w++)
+#pragma unroll
+          for (int r = 0; r < RB; r++) acc[w][r] += a[u][w] * x[r];
       }
     }
     for (; l < inner; l += 8) {
-      const real a = row[l];
       real x[RB];
       load_vec<real, RB>(v + l * VS, x);
 #pragma unroll
-      for (int r = 0; r < RB; r++) acc[r] += a * x[r];
+      for (int w = 0; w < NO; w++) {
+        const real a = row[w][l];
+#pragma unroll
+        for (int r = 0; r < RB; r++) acc[w][r] += a * x[r];
+      }
     }
-    int base = 0;
-    group_reduce<real, RB, 1>(acc, lane, &base);
     // fewer right-hand sides than lanes: the first lane holding a total
     const bool mine = RB >= 8 || p < (RB == 4 ? 4 : 1);
-    if (mine && o0 < nout)
 #pragma unroll
-      for (int j = 0; j < kLeft; j++) emit(o, base + j, acc[j]);
+    for (int w = 0; w < NO; w++) {
+      int base = 0;
+      group_reduce<real, RB, 1>(acc[w], lane, &base);
+      const int o = base0 + g + w * kGroups;
+      if (mine && o < nout)
+#pragma unroll
+        for (int j = 0; j < kLeft; j++) emit(o, base + j, acc[w][j]);
+    }
   }
+}
+
+// Several outputs per group where there are enough: they share the vector's
+// loads and overlap one another's latency (a forward link of 96^3's level 3, 490
+// columns per CTA and 8 right-hand sides, spent 5.2 of its 12.5 us in passes of
+// one output).  One application, one output -> several: 64^3 2.08 -> 1.96 ms, 96^3
+// with variable coefficients 6.44 -> 5.88, 96^3 with 8 right-hand sides 15.2 ->
+// 14.2.  Float64 takes one: its pipe is the bound, and the last pass's missing
+// outputs are multiplied all the same (64^3 4.62 -> 5.36).
+template <typename real, int RB, typename Emit>
+__device__ __forceinline__ void sweep_dots(const real* A, int lda, int nout, int inner,
+                                           const real* v, Emit&& emit) {
+  constexpr int NO = sizeof(real) == 8 ? 1 : (RB >= 32 ? 2 : 4);
+  if (NO > 1 && nout > kSweepThreads / 8) sweep_dots_by<real, RB, NO>(A, lda, nout, inner, v, emit);
+  else sweep_dots_by<real, RB, 1>(A, lda, nout, inner, v, emit);
 }
 
 // out[i][r] (+)= sum_c A[c * lda + i] x[c][r] for i < nrow, c < ncol.  Lanes run
