@@ -32,11 +32,86 @@ namespace {
 constexpr int TM = 64, TN = 64, TK = 16;
 constexpr int kMaxGridYZ = 65535;  // grid y/z limit: larger task lists are split
 
+template <typename real>
+struct alignas(4 * sizeof(real) > 16 ? 16 : 4 * sizeof(real)) Quad {
+  real v[4];
+};
+template <typename real>
+struct alignas(2 * sizeof(real)) Pair {
+  real v[2];
+};
+
+// One tile of gemm_gather: 16 S rows from i0, TN columns from j0.  The thread
+// (tx, ty) has rows tx + 16 p and columns 4 ty + q.
+template <typename real, int S, int KC>
+__device__ __forceinline__ void gather_tile(const GemmTask& tk, const real* __restrict__ A,
+                                            const real* __restrict__ Bbase, real* C, int M, int i0,
+                                            int j0, const int64_t* cp, const int* cst, real* As,
+                                            real* Bs) {
+  constexpr int PB = TN + 4;
+  const int N = tk.N, K = tk.K;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  real acc[S][4];
+#pragma unroll
+  for (int a = 0; a < S; a++)
+#pragma unroll
+    for (int b = 0; b < 4; b++) acc[a][b] = 0;
+  for (int l0 = 0; l0 < K; l0 += KC) {
+    const int lc = min(KC, K - l0);
+    // consecutive threads along rows of A, and along the gathered columns
+#pragma unroll
+    for (int h = 0; h < KC; h += 16) {
+      if (h >= lc) break;
+#pragma unroll
+      for (int u = 0; u < S; u++) {
+        const int i = tx + 16 * u, l = h + ty;
+        As[l * TM + i] =
+            (i0 + i < M && l < lc) ? A[i0 + i + (int64_t)(l0 + l) * tk.lda] : real(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int j = ty + 16 * u, l = h + tx;
+        Bs[l * PB + j] =
+            (l < lc && j0 + j < N) ? Bbase[cp[j] + (int64_t)(l0 + l) * cst[j]] : real(0);
+      }
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int l = 0; l < lc; l++) {
+      real a[S];
+#pragma unroll
+      for (int p = 0; p < S; p++) a[p] = As[l * TM + tx + 16 * p];
+      const Quad<real> b = *reinterpret_cast<const Quad<real>*>(Bs + l * PB + 4 * ty);
+#pragma unroll
+      for (int p = 0; p < S; p++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc[p][q] += a[p] * b.v[q];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < 4; q++)
+#pragma unroll
+    for (int p = 0; p < S; p++) {
+      const int gi = i0 + tx + 16 * p, gj = j0 + 4 * ty + q;
+      if (gi < M && gj < N) C[gi + (int64_t)gj * tk.ldc] = acc[p][q];
+    }
+}
+
 // rows of A (M), inner K and skip rule from the rank of the cluster:
 //   mode 0: M = task.M, K = task.K; skip when rank == m (untouched)
 //   mode 1: M = rank; skip when rank == 0 or rank == m
+//
+// Bound: the FP64 pipe in float64, latency of short tiles in float32.  The rows
+// go in equal tiles of a whole number of 16-row strips (S = 1 to 4), so a
+// cluster of 130 unknowns computes 144 rows and not 192, and a rank of 20
+// computes 32 and not 64; S is a template argument since a strip skipped inside
+// the product loop costs more than it saves (fill products 73 ms against 65).
+// Chunks of 32 and a vector read of the gathered operand as in the Schur
+// update.  Both products per factorization, before -> now: float64 64^3 115 ->
+// 77 ms, 96^3 40 -> 29, convection-diffusion 64^3 31 -> 23.
 template <typename real>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(real) == 8 ? 2 : 5)
 gemm_gather_kernel(const GemmTask* __restrict__ tasks, const real* __restrict__ Abase,
                    real* __restrict__ Cbase, const real* __restrict__ Bbase,
                    const Seg* __restrict__ segs, const int* __restrict__ rank) {
@@ -49,11 +124,13 @@ gemm_gather_kernel(const GemmTask* __restrict__ tasks, const real* __restrict__ 
     if (r == 0 || r == tk.K) return;
     M = r;
   }
-  const int N = tk.N, K = tk.K;
-  const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
-  if (i0 >= M || j0 >= N) return;
-  __shared__ real As[TK][TM + 1];
-  __shared__ real Bs[TK][TN + 1];
+  const int nt = (M + TM - 1) / TM, j0 = blockIdx.x * TN;
+  if ((int)blockIdx.y >= nt || j0 >= tk.N) return;
+  const int S = (M + 16 * nt - 1) / (16 * nt), i0 = blockIdx.y * 16 * S;
+  if (i0 >= M) return;
+  constexpr int KC = 32;
+  __shared__ __align__(16) real As[KC * TM];
+  __shared__ __align__(16) real Bs[KC * (TN + 4)];
   __shared__ int64_t cp[TN];
   __shared__ int cst[TN];
   // this tile's gathered columns: offset and stride, resolved once
@@ -61,51 +138,15 @@ gemm_gather_kernel(const GemmTask* __restrict__ tasks, const real* __restrict__ 
     seg_col(segs + tk.bcol, tk.nseg, j0 + threadIdx.x, &cp[threadIdx.x], &cst[threadIdx.x]);
   __syncthreads();
   const real* A = Abase + tk.A;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  real acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; a++)
-#pragma unroll
-    for (int b = 0; b < 4; b++) acc[a][b] = 0;
-  for (int l0 = 0; l0 < K; l0 += TK) {
-    // A tile: TM x TK, consecutive threads along rows
-    for (int e = threadIdx.x; e < TM * TK; e += 256) {
-      int i = e % TM, l = e / TM;
-      int gi = i0 + i, gl = l0 + l;
-      As[l][i] = (gi < M && gl < K) ? A[gi + (int64_t)gl * tk.lda] : real(0);
-    }
-    // B tile: TK x TN, consecutive threads along the gathered column
-    for (int e = threadIdx.x; e < TK * TN; e += 256) {
-      int l = e % TK, j = e / TK;
-      int gl = l0 + l, gj = j0 + j;
-      real v = 0;
-      if (gl < K && gj < N) v = Bbase[cp[j] + (int64_t)gl * cst[j]];
-      Bs[l][j] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int l = 0; l < TK; l++) {
-      real a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        a[q] = As[l][ty + 16 * q];
-        b[q] = Bs[l][tx + 16 * q];
-      }
-#pragma unroll
-      for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc[p][q] += a[p] * b[q];
-    }
-    __syncthreads();
-  }
   real* C = Cbase + tk.C;
-#pragma unroll
-  for (int p = 0; p < 4; p++)
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      int gi = i0 + ty + 16 * p, gj = j0 + tx + 16 * q;
-      if (gi < M && gj < N) C[gi + (int64_t)gj * tk.ldc] = acc[p][q];
-    }
+  if (S == 4)
+    gather_tile<real, 4, KC>(tk, A, Bbase, C, M, i0, j0, cp, cst, As, Bs);
+  else if (S == 3)
+    gather_tile<real, 3, KC>(tk, A, Bbase, C, M, i0, j0, cp, cst, As, Bs);
+  else if (S == 2)
+    gather_tile<real, 2, KC>(tk, A, Bbase, C, M, i0, j0, cp, cst, As, Bs);
+  else
+    gather_tile<real, 1, KC>(tk, A, Bbase, C, M, i0, j0, cp, cst, As, Bs);
 }
 
 // SplitMix64 output function (Steele, Lea, Flood 2014; Vigna's public
@@ -203,14 +244,6 @@ sketch_kernel(const SketchTask* __restrict__ tasks, const real* __restrict__ are
 // six CTAs per SM.  Updates per factorization, before -> now: 96^3 138 -> 83
 // ms, convection-diffusion 64^3 28 -> 18, float64 64^3 127 -> 111.  Fewer loads
 // in flight: four 92, two 103; six CTAs per SM with eight: 96 (spills).
-template <typename real>
-struct alignas(4 * sizeof(real) > 16 ? 16 : 4 * sizeof(real)) Quad {
-  real v[4];
-};
-template <typename real>
-struct alignas(2 * sizeof(real)) Pair {
-  real v[2];
-};
 template <typename real>
 __global__ void __launch_bounds__(256)
 schur_kernel(const SchurTask* __restrict__ tasks, const real* __restrict__ fac,
