@@ -4,7 +4,9 @@
 // V^T A_ss^{-1} U = 0, the sparsification rows T = [U V]^T A_ss^{-1}
 // (Eq. scaling), factor the fine block F = V^T A_ss^{-1} V (Eq. elim) and fold
 // its inverse factor into T.  One CTA per cluster of a colour class; all
-// clusters of the class run in one launch.
+// clusters of the class run in one launch.  SPD clusters of up to 256 unknowns
+// take the blocked kernel of kernels_spd.cu instead; here are the general ones,
+// larger SPD ones and the shared helpers.
 //
 // Matrices are column-major.  `real` is the storage/compute type of the
 // factorization (double in float64 mode, float in the mixed modes); squared

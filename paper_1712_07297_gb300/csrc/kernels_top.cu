@@ -7,7 +7,7 @@
 // launch of CTAs solves the panel, a launch updates the trailing lower
 // triangle), then the explicit inverse factor X = L^{-1} recursively: the
 // 64 x 64 diagonal blocks inverted in one launch, then X21 = -X22 (L21 X11)
-// per split, as matrix products.  The substitution sweeps apply X as dense
+// for every pair of a level at once, as matrix products.  The substitution sweeps apply X as dense
 // products.  Matrices are column-major in global memory.
 //
 // General (nonsymmetric) top (Sec. 6): recursive LU with partial pivoting
