@@ -1146,7 +1146,8 @@ struct SweepShape {
 // CTAs per SM).  One application, CTAs wanted / share: 2 / 104 KB takes 2.08
 // ms at 64^3 (float32, 1 right-hand side), 15.2 ms at 96^3 (8) and 7.2 ms at
 // 512^2 (124); 4 / 56 KB took 2.03, 16.0 and 11.8 ms, 4 / 150 KB 2.35, 16.0
-// and 7.7 ms.  The four-launch form took 6.4, 34.2 and 18.8 ms.
+// and 7.7 ms, all with one output per lane group in the products (several: 1.95,
+// 14.2 and 6.95 ms).  The four-launch form took 6.4, 34.2 and 18.8 ms.
 constexpr size_t kShare = 104 * 1024;
 template <typename real, int RB>
 SweepShape sweep_shape(bool fwd, int nids, int maxm, int maxnw, int nrhs) {
