@@ -470,6 +470,9 @@ __global__ void scatter_csr_kernel(const int64_t* __restrict__ dst, const double
 
 // The level-to-level copies sit between two sweeps that are programmatic
 // dependents of one another (kernels_apply.cu) and take part in the chain.
+// The kernel ahead still writes `src` when they start, so they make no promise
+// that it is read-only (no __restrict__: such loads may go through the
+// non-coherent cache) and read it from L2.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -491,28 +494,26 @@ void launch_pdl(void (*kernel)(KArgs...), int grid, cudaStream_t st, Args... arg
 }
 
 template <typename real>
-__global__ void gather_vec_kernel(const int64_t* __restrict__ idx, int64_t n,
-                                  const real* __restrict__ src, int64_t lds, real* __restrict__ dst,
-                                  int64_t ldd, int nrhs) {
+__global__ void gather_vec_kernel(const int64_t* __restrict__ idx, int64_t n, const real* src,
+                                  int64_t lds, real* dst, int64_t ldd, int nrhs) {
   pdl_begin();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * nrhs;
        e += (int64_t)gridDim.x * blockDim.x) {
     int64_t p = e % n;
     int r = (int)(e / n);
-    dst[p + r * ldd] = src[idx[p] + r * lds];
+    dst[p + r * ldd] = __ldcg(src + idx[p] + r * lds);
   }
 }
 
 template <typename real>
-__global__ void scatter_vec_kernel(const int64_t* __restrict__ idx, int64_t n,
-                                   const real* __restrict__ src, int64_t lds,
-                                   real* __restrict__ dst, int64_t ldd, int nrhs) {
+__global__ void scatter_vec_kernel(const int64_t* __restrict__ idx, int64_t n, const real* src,
+                                   int64_t lds, real* dst, int64_t ldd, int nrhs) {
   pdl_begin();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * nrhs;
        e += (int64_t)gridDim.x * blockDim.x) {
     int64_t p = e % n;
     int r = (int)(e / n);
-    dst[idx[p] + r * ldd] = src[p + r * lds];
+    dst[idx[p] + r * ldd] = __ldcg(src + p + r * lds);
   }
 }
 
