@@ -50,7 +50,7 @@ __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
 // runs in ascending order in one accumulator.  A thread's rows are strided so
 // that a warp reads consecutive ones.  C must not alias A or B.  (Staging 16
 // inner indices at a time instead took two barriers per chunk: 43 us for the
-// 128 x 128 x 128 product of [U V]^T A_ss^{-1} against 17.)
+// 128 x 128 x 128 product of [U V]^T A_ss^{-1} in shared memory against 17.)
 template <typename real, int RM, int RN>
 __device__ __forceinline__ void gemm_tiles(int M, int N, int K, const real* A, int ars, int acs,
                                            const real* B, int brs, int bcs, real* C, int ldc) {
@@ -87,10 +87,76 @@ __device__ __forceinline__ void gemm_tiles(int M, int N, int K, const real* A, i
   }
 }
 
+// The same for a transposed A in the workspace, float32: the rows a warp
+// multiplies are then a leading dimension apart, so 16 inner indices of 128 rows
+// at a time go through shared memory (As, kAtElems), read and written without
+// bank conflicts, and a warp multiplies four columns whose elements are the same
+// for all lanes.  Straight from memory these products were slower from 133
+// unknowns on, where [U V] leaves shared memory: [U V]^T A_ss^{-1} of all clusters
+// of 128^2 with leaf size 512 86 ms against 13, L^{-T} L^{-1} with the triangular
+// inverse before it 126 against 59, the whole step with leaf size 256
+// (convection-diffusion) 50 against 35.  (Float64 is bound by its pipe: 163 ms
+// straight for the first, 182 staged.)
+constexpr int kAtRows = 128, kAtInner = 16, kAtLd = kAtRows + 2, kAtElems = kAtInner * kAtLd;
+__device__ __forceinline__ void gemm_staged_at(int M, int N, int K, const float* A, int lda,
+                                               const float* B, int brs, int bcs, float* C, int ldc,
+                                               float* As) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int i0 = 0; i0 < M; i0 += kAtRows)
+    for (int j0 = 0; j0 < N; j0 += 4 * nw) {
+      const int jf = j0 + 4 * warp;
+      int bo[4];
+#pragma unroll
+      for (int c = 0; c < 4; c++) bo[c] = min(jf + c, N - 1) * bcs;
+      float acc[4][4];
+#pragma unroll
+      for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[r][c] = 0;
+      for (int l0 = 0; l0 < K; l0 += kAtInner) {
+        const int lc = min(kAtInner, K - l0);
+        for (int e = threadIdx.x; e < kAtRows * kAtInner; e += blockDim.x) {
+          const int l = e % kAtInner, i = e / kAtInner;
+          As[l * kAtLd + i] = (i0 + i < M && l < lc) ? A[l0 + l + (i0 + i) * lda] : 0.f;
+        }
+        __syncthreads();
+        if (jf < N) {
+#pragma unroll 8
+          for (int l = 0; l < lc; l++) {
+            float a[4], b[4];
+#pragma unroll
+            for (int r = 0; r < 4; r++) a[r] = As[l * kAtLd + lane + 32 * r];
+#pragma unroll
+            for (int c = 0; c < 4; c++) b[c] = B[bo[c] + (l0 + l) * brs];
+#pragma unroll
+            for (int r = 0; r < 4; r++)
+#pragma unroll
+              for (int c = 0; c < 4; c++) acc[r][c] += a[r] * b[c];
+          }
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+          if (i0 + lane + 32 * r < M && jf + c < N)
+            C[i0 + lane + 32 * r + (int64_t)(jf + c) * ldc] = acc[r][c];
+    }
+}
+
 template <typename real>
 __device__ void cta_gemm(int M, int N, int K, const real* A, int lda, bool ta, const real* B,
                          int ldb, bool tb, real* C, int ldc) {
   const int ars = ta ? lda : 1, acs = ta ? 1 : lda, brs = tb ? ldb : 1, bcs = tb ? 1 : ldb;
+  if constexpr (sizeof(real) == 4) {
+    if (ta && !__isShared(A)) {  // uniform
+      __shared__ float As[kAtElems];
+      gemm_staged_at(M, N, K, A, lda, B, brs, bcs, C, ldc, As);
+      __syncthreads();
+      return;
+    }
+  }
   if (M * N >= 12 * (int)blockDim.x)
     gemm_tiles<real, 4, 4>(M, N, K, A, ars, acs, B, brs, bcs, C, ldc);
   else
