@@ -19,9 +19,9 @@
 //
 // The dense top (one cluster, nothing but a triangular T' of thousands of
 // unknowns) has kernels of its own that stream the triangle once from HBM.
-// Clusters too large for the shared-memory vectors of the fused kernels
-// (leaf sizes in the thousands) take the unfused ones: fwd_t, fwd_nbr,
-// bwd_part, bwd_z, bwd_t.
+// Clusters too large for the shared-memory vectors of the fused kernels, and
+// large ones with many right-hand sides (kManyRhs), take the unfused ones:
+// fwd_t, fwd_nbr, bwd_part, bwd_z, bwd_t.
 #include <algorithm>
 #include <cooperative_groups.h>
 #include <type_traits>
@@ -536,6 +536,9 @@ __device__ __forceinline__ void sweep_dots_by(const real* A, int lda, int nout, 
   constexpr int kGroups = kSweepThreads / 8;
   const int lane = threadIdx.x & 31, p = threadIdx.x & 7, g = threadIdx.x >> 3;
   for (int base0 = 0; base0 < nout; base0 += kGroups * NO) {
+    // (a warp whose outputs are all missing from the last pass leaves the pipes
+    // to the others)
+    if (base0 + (g & ~3) >= nout) break;
     const real* row[NO];
 #pragma unroll
     for (int w = 0; w < NO; w++) row[w] = A + min(base0 + g + w * kGroups, nout - 1) * lda;
@@ -1212,11 +1215,22 @@ bool try_sweep(bool fwd, const ApplyRec* recs, const int* ids, int nids, int max
   return true;
 }
 
+// Large clusters with many right-hand sides take the unfused kernels: a link's
+// latency no longer counts, and each group of right-hand sides stages the class's
+// operators anew and multiplies by slices of T' that leave lanes idle.  One
+// application with 128 right-hand sides, fused -> these clusters unfused:
+// float64, clusters of 183 (36^3) 40.3 -> 35.9 ms, 160 equal, 144 22.2 -> 22.9; float32
+// (whose fused groups of 32 end at 256 unknowns) 350 (150 x 148) 3.76 -> 2.44, 264
+// (33 x 32^2) 6.23 -> 4.93, 256 equal, 184 5.54 -> 5.86.  With 64: 183 21.9 -> 20.7, 256
+// (float64) 4.67 -> 4.86, 264 3.62 -> 3.64; with 32 the fused ones win throughout.
+constexpr int kManyRhs = 64, kWideF64 = 160, kWideF32 = 256;
+
 template <typename real>
 bool sweep_class(bool fwd, const ApplyRec* recs, const int* ids, int nids, int maxm, int maxnw,
                  const real* fac, const int64_t* vmap, real* y, int64_t ldy, int nrhs,
                  cudaStream_t st) {
   if (nids > 65535 || nrhs > 65535) return false;
+  if (nrhs > kManyRhs && maxm > (sizeof(real) == 8 ? kWideF64 : kWideF32)) return false;
   const auto fits = [&](int rb) {
     return (int64_t)nids * kSweepMaxCl * ((nrhs + rb - 1) / rb) <= kAtOnce;
   };
