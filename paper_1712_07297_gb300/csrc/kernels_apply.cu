@@ -905,15 +905,15 @@ bwd_sweep_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
 // ---------------------------------------------------------------------------
 // The dense top: z = T' y and y = T_R'^T z with T' and T_R'^T n x n, read
 // once from HBM (lower triangular but for the permuted columns of a general
-// T': tri).  A thread-block cluster of kTopCl CTAs shares 64 rows (forward)
+// T': tri).  A thread-block cluster of CL CTAs shares 64 rows (forward)
 // or 32 columns (backward), each CTA a stretch of the other index, and adds
 // the CTAs' sums through distributed shared memory: 93 x 8 and 185 x 8 CTAs
 // for 5,909 unknowns keep enough loads in flight for the HBM rate, which one
 // CTA per 64 rows (93 CTAs, four loads each) did not.
 // ---------------------------------------------------------------------------
-constexpr int kTopCl = 8, kTopRows = 64, kTopCols = 32, kTopChunk = 256;
+constexpr int kTopRows = 64, kTopCols = 32, kTopChunk = 256;
 
-template <typename real, int RB>
+template <typename real, int RB, int CL>
 __global__ void __launch_bounds__(kSweepThreads)
 fwd_top_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
                const real* __restrict__ fac, const real* y, real* z, int64_t ldy, int nrhs,
@@ -929,7 +929,7 @@ fwd_top_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
   const int i0 = ((int)gridDim.y - 1 - (int)blockIdx.y) * kTopRows;
   const int r0 = blockIdx.z * RB, nr = min(RB, nrhs - r0);
   const int cols = tri ? min(n, i0 + kTopRows) : n;
-  const int per = (cols + kTopCl - 1) / kTopCl;
+  const int per = (cols + CL - 1) / CL;
   const int l0 = min(cols, cr * per), l1 = min(cols, l0 + per);
   const int ii = threadIdx.x % kTopRows, part = threadIdx.x / kTopRows;
   const int i = min(i0 + ii, n - 1);
@@ -969,17 +969,17 @@ fwd_top_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
     __syncthreads();
   }
   cl.sync();
-  for (int e = cr * kSweepThreads + threadIdx.x; e < kTopRows * nr; e += kTopCl * kSweepThreads) {
+  for (int e = cr * kSweepThreads + threadIdx.x; e < kTopRows * nr; e += CL * kSweepThreads) {
     const int a = e % kTopRows;
     real s = 0;
 #pragma unroll
-    for (int q = 0; q < kTopCl; q++) s += cl.map_shared_rank(red, q)[e];
+    for (int q = 0; q < CL; q++) s += cl.map_shared_rank(red, q)[e];
     if (i0 + a < n) z[rc.voff + i0 + a + (int64_t)(r0 + e / kTopRows) * ldy] = s;
   }
   cl.sync();
 }
 
-template <typename real, int RB>
+template <typename real, int RB, int CL>
 __global__ void __launch_bounds__(kSweepThreads)
 bwd_top_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
                const real* __restrict__ fac, real* y, const real* z, int64_t ldy, int nrhs) {
@@ -994,7 +994,7 @@ bwd_top_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
   const int i0 = blockIdx.y * kTopCols;
   const int r0 = blockIdx.z * RB, nr = min(RB, nrhs - r0);
   // rows i0.. only: T_R'^T is lower triangular
-  const int rows = n - i0, per = (rows + kTopCl - 1) / kTopCl;
+  const int rows = n - i0, per = (rows + CL - 1) / CL;
   const int l0 = min(n, i0 + cr * per), l1 = min(n, l0 + per);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const real* T = fac + (rc.sym ? rc.T : rc.TR);
@@ -1043,11 +1043,11 @@ bwd_top_kernel(const ApplyRec* __restrict__ recs, const int* __restrict__ ids,
       if (lane == 0) red[r * kTopCols + warp * kPer + w] = v;
     }
   cl.sync();
-  for (int e = cr * kSweepThreads + threadIdx.x; e < kTopCols * nr; e += kTopCl * kSweepThreads) {
+  for (int e = cr * kSweepThreads + threadIdx.x; e < kTopCols * nr; e += CL * kSweepThreads) {
     const int a = e % kTopCols;
     real s = 0;
 #pragma unroll
-    for (int q = 0; q < kTopCl; q++) s += cl.map_shared_rank(red, q)[e];
+    for (int q = 0; q < CL; q++) s += cl.map_shared_rank(red, q)[e];
     if (i0 + a < n) y[rc.voff + i0 + a + (int64_t)(r0 + e / kTopCols) * ldy] = s;
   }
   cl.sync();
@@ -1245,16 +1245,37 @@ bool sweep_class(bool fwd, const ApplyRec* recs, const int* ids, int nids, int m
   return go(std::integral_constant<int, 8>{});
 }
 
+// CTAs per cluster of a top of n unknowns whose launch has `tiles` clusters: 8,
+// fewer when the chip stays full without them and a CTA's stretch would be
+// shorter than a staged chunk, as in a small top with many right-hand sides: its
+// start and the exchange then cost more than its products (float64, one
+// application with 256 right-hand sides, 8 CTAs -> the rule: 400 unknowns 0.52 ->
+// 0.29 ms, 1,000 1.42 -> 0.83).
+int top_ctas(int n, int64_t tiles) {
+  int CL = kSweepMaxCl;
+  while (CL > 2 && n < CL * kTopChunk && tiles * CL / 2 >= kAtOnce) CL /= 2;
+  return CL;
+}
+
 template <typename real, int RB>
 void launch_top(bool fwd, const ApplyRec* recs, const int* ids, int n, bool sym, const real* fac,
                 real* y, real* z, int64_t ldy, int nrhs, cudaStream_t st) {
-  const int nz = (nrhs + RB - 1) / RB;
-  if (fwd)
-    launch_pdl(fwd_top_kernel<real, RB>, dim3(kTopCl, (n + kTopRows - 1) / kTopRows, nz), kTopCl, 0,
-               st, recs, ids, fac, y, z, ldy, nrhs, sym ? 1 : 0);
-  else
-    launch_pdl(bwd_top_kernel<real, RB>, dim3(kTopCl, (n + kTopCols - 1) / kTopCols, nz), kTopCl, 0,
-               st, recs, ids, fac, y, z, ldy, nrhs);
+  const int nz = (nrhs + RB - 1) / RB, per = fwd ? kTopRows : kTopCols, nt = (n + per - 1) / per;
+  const auto go = [&](auto cl) {
+    constexpr int CL = decltype(cl)::value;
+    const dim3 grid(CL, nt, nz);
+    if (fwd)
+      launch_pdl(fwd_top_kernel<real, RB, CL>, grid, CL, 0, st, recs, ids, fac, y, z, ldy, nrhs,
+                 sym ? 1 : 0);
+    else
+      launch_pdl(bwd_top_kernel<real, RB, CL>, grid, CL, 0, st, recs, ids, fac, y, z, ldy, nrhs);
+  };
+  if constexpr (RB >= 8) {  // (fewer right-hand sides leave too few tiles)
+    const int CL = top_ctas(n, (int64_t)nt * nz);
+    if (CL == 2) return go(std::integral_constant<int, 2>{});
+    if (CL == 4) return go(std::integral_constant<int, 4>{});
+  }
+  go(std::integral_constant<int, kSweepMaxCl>{});
 }
 
 }  // namespace

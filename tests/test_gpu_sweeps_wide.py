@@ -1,7 +1,8 @@
 """The substitution sweeps with many right-hand sides: on both sides of the
 sizes where large clusters leave the fused kernels (160 unknowns in float64, 256
-in float32, more than 64 right-hand sides), and clusters whose forward step is
-fused and whose backward step is not, against the CPU oracle.
+in float32, more than 64 right-hand sides), clusters whose forward step is fused
+and whose backward step is not, and small dense tops whose clusters of CTAs shrink,
+against the CPU oracle.
 
 Bars: float64 within 1e-10 of the oracle's M^{-1} b, column by column; float32
 against the same factorization's one-column applications, where only the order of
@@ -25,6 +26,9 @@ CASES = {
     "m250": ((50, 40), 250, 0),
     "m256": ((16, 16, 16), 256, 0),
     "m264": ((33, 16, 8), 264, 0),
+    "top272": ((17, 16), 64, 272),
+    "top400": ((20, 20), 64, 400),
+    "top1000": ((10, 10, 10), 64, 1000),
 }
 
 
