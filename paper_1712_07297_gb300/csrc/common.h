@@ -266,7 +266,7 @@ struct Launch {
   // the same for an SPD factorization whose pivoted QRs have run (or have no
   // columns); false, nothing launched, for clusters above its limit
   static bool prep_spd(const PrepTask* tasks_dev, int ntask, real* arena, real* fac, real* ws,
-                       double* wsd, int* rank, int maxm, DevError* err, int level,
+                       double* wsd, int* rank, int maxm, DevError* err, int level, long long* dbg,
                        cudaStream_t st);
   // thread-block-cluster pivoted QR: cluster size for the largest task (0 =
   // does not fit), its dynamic shared memory, and the launch

@@ -1234,7 +1234,7 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
     for (auto& pt : prep) spd = spd && (pt.qr == 2 || pt.ncolG == 0);
     timed_lv(h, "prep", level, 1, [&] {
       if (spd && Launch<real>::prep_spd(d_prep, nt, arena, fac, ws, h->wsd.as<double>(), rank,
-                                        maxm, h->d_err.as<DevError>(), level, h->st))
+                                        maxm, h->d_err.as<DevError>(), level, dbg, h->st))
         return;
       Launch<real>::prep(d_prep, nt, arena, fac, ws,
                          h->wsd.as<double>(), d_segs, rank, pivd, fpiv, eps, sym ? 1 : 0,

@@ -225,8 +225,9 @@ __host__ __device__ inline int scratch_elems(int n) {
 
 // A (n x n, lower triangle) becomes L^{-1} of its Cholesky factor L, zeros
 // above the diagonal; false (for every thread) when a pivot is not positive.
-template <typename real>
-__device__ bool chol_inverse(int n, real* A, int ld, real* tmp, int* flag) {
+// factored() is called between the factorization and the rest of the inverse.
+template <typename real, typename Mark>
+__device__ bool chol_inverse(int n, real* A, int ld, real* tmp, int* flag, Mark&& factored) {
   for (int p = 0; p < n; p += NB) {
     const int nb = min(NB, n - p), rest = n - p - nb;
     real* D = A + p + p * ld;
@@ -255,6 +256,7 @@ __device__ bool chol_inverse(int n, real* A, int ld, real* tmp, int* flag) {
   for (int j = warp_id(); j < n; j += NT / 32)
     for (int i = lane_id(); i < j; i += 32) A[i + j * ld] = 0;
   __syncthreads();
+  factored();
   tri_inv_levels<real>(n, A, ld, tmp);
   return true;
 }
@@ -401,12 +403,19 @@ template <typename real>
 __global__ void __launch_bounds__(NT)
 prep_spd_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena,
                 real* __restrict__ fac, real* __restrict__ ws_all, double* __restrict__ wsd_all,
-                int* rank, int smem_mats, int smem_m, DevError* err, int level) {
+                int* rank, int smem_mats, int smem_m, DevError* err, int level, long long* dbg) {
   extern __shared__ __align__(16) unsigned char spd_smem[];
   __shared__ real vbuf[2 * 128];
   __shared__ real tbuf[2];
   __shared__ int flag;
   const PrepTask tk = tasks[blockIdx.x];
+  // optional per-phase clock stamps (profiling), the general kernel's
+  // checkpoints: 0 -> 1 factor, 3 -> 4 inverse, -> 5 bases, -> 6 Z, -> 7 F and T'
+  long long* stamp = dbg ? dbg + (int64_t)blockIdx.x * 8 : nullptr;
+  const auto mark = [&](int i) {
+    if (stamp && threadIdx.x == 0) stamp[i] = clock64();
+  };
+  mark(0);
   const int m = tk.m;
   const int64_t mm = (int64_t)m * m, reg = (int64_t)(smem_m | 1) * smem_m;
   real* sm = reinterpret_cast<real*>(spd_smem);
@@ -432,10 +441,14 @@ prep_spd_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena,
   for (int j = warp; j < m; j += W)
     for (int i = lane; i < m; i += 32) R1[i + j * ld1] = arena[tk.a_ss + i + (int64_t)j * tk.ld];
   __syncthreads();
-  if (!chol_inverse<real>(m, R1, ld1, tmp, &flag)) {
+  if (!chol_inverse<real>(m, R1, ld1, tmp, &flag, [&] {
+        mark(1);
+        mark(3);
+      })) {
     fail<real>(err, tk.s, level, rank, m);
     return;
   }
+  mark(4);
   if (k == m) return;  // untouched: all unknowns coarse, E_s = I
   if (k == 0) {  // E_s = I: T' = L^{-1}
     for (int j = warp; j < m; j += W)
@@ -504,14 +517,16 @@ prep_spd_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena,
                                   });
   }
   __syncthreads();
+  mark(5);
   // ---- Z = Li V (R2), F = Z^T Z (R3) and the inverse of its factor
   product<real, kFrom0, kToRow>(m, f, m, R1, 1, ld1, R3 + k * ld3, 1, ld3, false, 0,
                                 [&](int i, int j, real v) { R2[i + j * ld2] = v; });
   __syncthreads();
+  mark(6);
   product<real, kFrom0, kToEnd>(f, f, m, R2, ld2, 1, R2, 1, ld2, true, 0,
                                 [&](int i, int j, real v) { R3[i + j * ld3] = v; });
   __syncthreads();
-  if (!chol_inverse<real>(f, R3, ld3, tmp, &flag)) {
+  if (!chol_inverse<real>(f, R3, ld3, tmp, &flag, [] {})) {
     fail<real>(err, tk.s, level, rank, m);
     return;
   }
@@ -528,6 +543,7 @@ prep_spd_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena,
   }
   product<real, kFromCol, kToEnd>(f, m, m, R2, ld2, 1, R1, 1, ld1, false, 0,
                                   [&](int i, int j, real v) { T[k + i + (int64_t)j * m] = v; });
+  mark(7);
   // C into the (s,s) block (coarse part); last: A_ss was copied
   real* ss = arena + tk.a_ss;
   for (int j = warp; j < k; j += W)
@@ -549,7 +565,7 @@ chol_inv_leaf_kernel(const real* __restrict__ A, int64_t lda, real* __restrict__
   for (int j = warp_id(); j < n; j += NT / 32)
     for (int i = lane_id(); i < n; i += 32) R[i + j * ld] = A[i + (int64_t)j * lda];
   __syncthreads();
-  if (!chol_inverse<real>(n, R, ld, tmp, &flag)) {
+  if (!chol_inverse<real>(n, R, ld, tmp, &flag, [] {})) {
     if (threadIdx.x == 0 && atomicCAS(&err->code, 0, (int)HSOLVE_ERR_NOT_SPD) == 0) {
       err->cluster = 0;
       err->level = level;
@@ -578,7 +594,7 @@ void chol_inv_leaf(float* A, int64_t lda, float* X, int64_t ldx, int n, DevError
 template <typename real>
 bool Launch<real>::prep_spd(const PrepTask* tasks, int ntask, real* arena, real* fac, real* ws,
                             double* wsd, int* rank, int maxm, DevError* err, int level,
-                            cudaStream_t st) {
+                            long long* dbg, cudaStream_t st) {
   if (maxm > kMaxM) return false;
   if (ntask <= 0) return true;
   const size_t budget = 224 * 1024;
@@ -594,13 +610,13 @@ bool Launch<real>::prep_spd(const PrepTask* tasks, int ntask, real* arena, real*
   (void)limit_set;
   count_launch();
   prep_spd_kernel<real><<<ntask, NT, mats * one + fix, st>>>(tasks, arena, fac, ws, wsd, rank, mats,
-                                                            maxm, err, level);
+                                                            maxm, err, level, dbg);
   return true;
 }
 
 template bool Launch<float>::prep_spd(const PrepTask*, int, float*, float*, float*, double*, int*,
-                                      int, DevError*, int, cudaStream_t);
+                                      int, DevError*, int, long long*, cudaStream_t);
 template bool Launch<double>::prep_spd(const PrepTask*, int, double*, double*, double*, double*,
-                                       int*, int, DevError*, int, cudaStream_t);
+                                       int*, int, DevError*, int, long long*, cudaStream_t);
 
 }  // namespace hs
