@@ -1200,7 +1200,10 @@ void factor_level(hsolve_handle* h, FLevel& FL, real* arena, int level, double e
                                 h->st));
         d_prep = reinterpret_cast<const PrepTask*>(h->blob3.as<char>() + o3_prep);
         const int* d_ord = reinterpret_cast<const int*>(h->blob3.as<char>() + o3_ord);
-        timed_lv(h, "qr_cluster", level, 1, [&] {
+        int groups = 0;  // launches: tasks of one form and cluster size share one
+        for (size_t i = 0; i < at.size(); i++)
+          groups += i == 0 || at[i][0] != at[i - 1][0] || at[i][1] != at[i - 1][1];
+        timed_lv(h, "qr_cluster", level, groups, [&] {
           for (size_t i = 0, e = 0; i < at.size(); i = e) {
             int nzm = 1;
             for (e = i; e < at.size() && at[e][0] == at[i][0] && at[e][1] == at[i][1]; e++)
