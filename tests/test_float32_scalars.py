@@ -1,0 +1,74 @@
+"""The float32 scalars of the pivoted QRs, on the host, against float64: the head and
+tau of a reflector are the float64 ones rounded once (within 0.501 ulp) wherever that
+is a finite float, columns of norms up to the square root of the largest float
+included."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+PKG = os.path.join(ROOT, "paper_1712_07297_gb300")
+
+SOURCE = """
+#include "common.h"
+extern "C" void run(long n, const float* r2, const float* x0, float* head, float* tau) {
+  for (long i = 0; i < n; i++) hs::householder_scalars(r2[i], x0[i], head + i, tau + i);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    d = tmp_path_factory.mktemp("scalars")
+    (d / "s.cu").write_text(SOURCE)
+    subprocess.run([nvcc, "-std=c++17", "-O2", "-shared", "-Xcompiler", "-fPIC", "-gencode",
+                    "arch=compute_103a,code=sm_103a", "--expt-relaxed-constexpr",
+                    "-I" + os.path.join(PKG, "csrc"), "-I" + os.path.join(ROOT, "include"),
+                    "-o", str(d / "s.so"), str(d / "s.cu")], check=True)
+    fn = C.CDLL(str(d / "s.so"), mode=os.RTLD_LAZY).run
+    fn.argtypes = [C.c_long] + [C.c_void_p] * 4
+
+    def call(r2, x0):
+        out = [np.empty_like(r2) for _ in range(2)]
+        fn(len(r2), r2.ctypes.data, x0.ctypes.data, *[o.ctypes.data for o in out])
+        return out
+
+    return call
+
+
+def _columns(lo, hi, n=400_000):
+    rng = np.random.default_rng(5)
+    r2 = (2.0 ** rng.uniform(lo, hi, n)).astype(np.float32)
+    part = np.where(rng.random(n) < 0.3, 2.0 ** rng.uniform(-40, 0, n), rng.random(n))
+    x0 = (np.sqrt(r2.astype(np.float64)) * part * rng.choice([-1, 1], n)).astype(np.float32)
+    x0[:100] = 0.0
+    return r2, x0
+
+
+@pytest.mark.parametrize("lo,hi", [(-30, 30), (-120, -60), (60, 127.99), (-148, -120)])
+def test_reflector_scalars(run, lo, hi):
+    r2, x0 = _columns(lo, hi)
+    head, tau = run(r2, x0)
+    r, x = np.sqrt(r2.astype(np.float64)), x0.astype(np.float64)
+    for got, want in ((head, np.where(x >= 0, x + r, x - r)), (tau, 1.0 / (r * (r + np.abs(x))))):
+        with np.errstate(over="ignore"):
+            w32 = want.astype(np.float32)
+        fin = np.isfinite(w32)
+        assert np.array_equal(np.isinf(got), ~fin)
+        err = np.abs(got[fin].astype(np.float64) - want[fin]) / np.spacing(np.abs(w32[fin])).astype(np.float64)
+        # (a tau below the normal floats is rounded twice: once more when scaled)
+        bar = np.where(np.abs(want[fin]) < 2.0 ** -126, 0.7505, 0.501)
+        assert (err <= bar).all(), (lo, hi, (err - bar).max())
+        normal = np.abs(w32[fin]) >= 2.0 ** -126
+        assert (got[fin] != w32[fin])[normal].mean() < 1e-4
+
+
+def test_no_column(run):
+    z = np.zeros(2, np.float32)
+    head, tau = run(z, z)
+    assert not head.any() and not tau.any()
