@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <mutex>
 #include <cstddef>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -132,6 +133,25 @@ __host__ __device__ __forceinline__ void householder_scalars(float r2, float x0,
   *tau = fmaf(t0, fmaf(-q, t0, 1.f) - ql * t0, t0) * s * s;
   *head = copysignf(h + hl, x0s >= 0.f ? 1.f : -1.f) *
           (s < 1.f ? 0x1p40f : (s > 1.f ? 0x1p-40f : 1.f));
+}
+
+// Near-ties of the float32 pivot search: squared norms carry ~1e-7 relative
+// rounding, so ties of exact arithmetic are recognised within 1e-5 of the
+// largest, M.  The smallest float that is not below (1 - 1e-5) M, the product in
+// a pair of floats: a float32 norm compares with it as with the float64 product.
+__host__ __device__ __forceinline__ float tie_band(float M) {
+  constexpr double c = 1.0 - 1e-5;
+  constexpr float ch = (float)c, cl = (float)(c - (double)(float)c);
+  const float p = M * ch;
+  const float lo = fmaf(M, cl, fmaf(M, ch, -p));  // (1 - 1e-5) M = p + lo
+  float b = p + lo;
+  if (lo - (b - p) > 0.f) {  // rounded down: one float up
+    unsigned u;
+    memcpy(&u, &b, sizeof(u));
+    u++;
+    memcpy(&b, &u, sizeof(u));
+  }
+  return b;
 }
 #endif
 

@@ -63,9 +63,7 @@ struct NormKey<float> {  // non-negative floats order as their bit patterns
   static __device__ __forceinline__ type warp_max(type k) {
     return __reduce_max_sync(0xffffffffu, k);
   }
-  // near-ties of the pivot search: squared norms carry ~1e-7 relative
-  // rounding, so ties of exact arithmetic are recognised within 1e-5
-  static __device__ __forceinline__ float band(float M) { return M * (1.0f - 1e-5f); }
+  static __device__ __forceinline__ float band(float M) { return tie_band(M); }
   // the largest float x with x <= v
   static __device__ __forceinline__ float floor_of(double v) { return __double2float_rd(v); }
 };

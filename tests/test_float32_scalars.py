@@ -1,7 +1,8 @@
 """The float32 scalars of the pivoted QRs, on the host, against float64: the head and
 tau of a reflector are the float64 ones rounded once (within 0.501 ulp) wherever that
 is a finite float, columns of norms up to the square root of the largest float
-included."""
+included, and the near-tie threshold is the smallest float not below the float64
+product."""
 import ctypes as C
 import os
 import shutil
@@ -15,8 +16,12 @@ PKG = os.path.join(ROOT, "paper_1712_07297_gb300")
 
 SOURCE = """
 #include "common.h"
-extern "C" void run(long n, const float* r2, const float* x0, float* head, float* tau) {
-  for (long i = 0; i < n; i++) hs::householder_scalars(r2[i], x0[i], head + i, tau + i);
+extern "C" void run(long n, const float* r2, const float* x0, float* head, float* tau,
+                    float* band) {
+  for (long i = 0; i < n; i++) {
+    hs::householder_scalars(r2[i], x0[i], head + i, tau + i);
+    band[i] = hs::tie_band(r2[i]);
+  }
 }
 """
 
@@ -31,10 +36,10 @@ def run(tmp_path_factory):
                     "-I" + os.path.join(PKG, "csrc"), "-I" + os.path.join(ROOT, "include"),
                     "-o", str(d / "s.so"), str(d / "s.cu")], check=True)
     fn = C.CDLL(str(d / "s.so"), mode=os.RTLD_LAZY).run
-    fn.argtypes = [C.c_long] + [C.c_void_p] * 4
+    fn.argtypes = [C.c_long] + [C.c_void_p] * 5
 
     def call(r2, x0):
-        out = [np.empty_like(r2) for _ in range(2)]
+        out = [np.empty_like(r2) for _ in range(3)]
         fn(len(r2), r2.ctypes.data, x0.ctypes.data, *[o.ctypes.data for o in out])
         return out
 
@@ -53,7 +58,7 @@ def _columns(lo, hi, n=400_000):
 @pytest.mark.parametrize("lo,hi", [(-30, 30), (-120, -60), (60, 127.99), (-148, -120)])
 def test_reflector_scalars(run, lo, hi):
     r2, x0 = _columns(lo, hi)
-    head, tau = run(r2, x0)
+    head, tau, _ = run(r2, x0)
     r, x = np.sqrt(r2.astype(np.float64)), x0.astype(np.float64)
     for got, want in ((head, np.where(x >= 0, x + r, x - r)), (tau, 1.0 / (r * (r + np.abs(x))))):
         with np.errstate(over="ignore"):
@@ -70,5 +75,15 @@ def test_reflector_scalars(run, lo, hi):
 
 def test_no_column(run):
     z = np.zeros(2, np.float32)
-    head, tau = run(z, z)
+    head, tau, _ = run(z, z)
     assert not head.any() and not tau.any()
+
+
+@pytest.mark.parametrize("lo,hi", [(-90, 127.9)])
+def test_tie_threshold(run, lo, hi):
+    r2, x0 = _columns(lo, hi)
+    band = run(r2, x0)[2].astype(np.float64)
+    want = (1.0 - 1e-5) * r2.astype(np.float64)
+    below = np.nextafter(band.astype(np.float32), np.float32(0)).astype(np.float64)
+    slack = want * 2.0 ** -47
+    assert (band >= want - slack).all() and (below < want + slack).all()
