@@ -1,8 +1,9 @@
-"""The per-cluster kernels, Cholesky and LU, at exact cluster sizes around their
-blocks of 32, their register tiles and the limit of 256 unknowns, and where their
-operands leave shared memory (general float32: one of the three from 133 unknowns,
-the second from 163, the last from 230), against the CPU oracle.  A grid of m 2^d
-unknowns bisects into clusters of exactly m, which the test asserts.
+"""The per-cluster kernels, Cholesky and LU, and the gathered products at exact
+cluster sizes: around the blocks of 32, the register tiles, the row strips of 16 and
+the limit of 256 unknowns, and where the operands of the general kernel leave shared
+memory (float32: one of the three from 133 unknowns, the second from 163, the last
+from 230), against the CPU oracle.  A grid of m 2^d unknowns bisects into clusters
+of exactly m, which the test asserts.
 
 Bars: float64 ranks equal (Cholesky) and M^{-1} b within 1e-10 of the oracle's,
 the bar of the parity tests; float32 at the oracle's ranks within 8 u kappa(A) of
@@ -19,8 +20,9 @@ from oracle import hsolver as H  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [((31, 32), 31), ((32, 32), 32), ((33, 32), 33), ((64, 32), 64), ((65, 32), 65),
-         ((97, 32), 97), ((127, 16), 127), ((64, 32), 128), ((16, 16, 8), 128), ((129, 16), 129),
+SIZES = [((16, 32), 16), ((17, 32), 17), ((48, 32), 48), ((49, 32), 49), ((31, 32), 31),
+         ((32, 32), 32), ((33, 32), 33), ((64, 32), 64), ((65, 32), 65), ((97, 32), 97),
+         ((127, 16), 127), ((64, 32), 128), ((16, 16, 8), 128), ((129, 16), 129),
          ((133, 16), 133), ((163, 16), 163), ((230, 8), 230), ((255, 8), 255), ((64, 32), 256),
          ((16, 16, 8), 256), ((257, 8), 257), ((60, 40), 300)]
 
