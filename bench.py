@@ -211,19 +211,25 @@ class ClockSampler:
                 "samples": len(self.samples)}
 
 
-def _traffic(kernel, workload, nclu, launches):
+def _traffic(kernel, workload, nclu, launches, spd=False):
     """DRAM bytes per launch of the dominant kernel from its committed ncu
     summary under profiles/: a figure captured on this workload
     ("traffic_bytes_per_launch(<kernel>, <workload>): N"), else a per-cluster
     figure measured on a smaller case and scaled by the clusters a launch
     processes here ("traffic_bytes_per_cluster: N" in the kernel's own
-    summary); None when no summary gives one."""
+    summary); None when no summary gives one.  A phase of a symmetric
+    factorization (spd) launches several kernels (prep_spd_kernel and
+    prep_kernel; qr_reg_kernel and qr_cluster_kernel; schur_kernel and
+    schur_targets_kernel): its figure is the average over them,
+    "traffic_bytes_per_launch(spd_<phase>, <workload>): N"."""
     import glob
     import re
     names = {"schur": "schur_kernel", "prep": "prep_kernel", "qr_cluster": "qr_cluster_kernel"}
     stem = names.get(kernel)
     if not stem:
         return None
+    if spd:
+        stem = "spd_" + kernel
     for f in sorted(glob.glob(os.path.join(ROOT, "profiles", "*.md"))):
         txt = open(f).read()
         m = re.search(r"traffic_bytes_per_launch\(%s, %s\):\s*(\d+)" % (stem, re.escape(workload)),
@@ -378,7 +384,8 @@ def run_gpu(args, rank, world):
     else:
         peak, bound, psrc = probes["fp32_simt"], "alu", "measured: cuBLAS SGEMM 8192^3, TF32 off"
     roof = {"bound": bound, "kernel": dom, "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-            "frac": ach / peak, "traffic": _traffic(dom, args.workload, nclu_done, nl_dom),
+            "frac": ach / peak, "traffic": _traffic(dom, args.workload, nclu_done, nl_dom,
+                                                prob.spd),
             "launches_per_step": nl_dom, "ms_per_step": ms_dom,
             "work": "algorithmic float32 flops per step from the factorization's ranks and "
                     "sizes: prep 2/3 m^3 + 6 m^2 k + 2 m^3, Schur 2 f nw^2, QR 4 m c k",
