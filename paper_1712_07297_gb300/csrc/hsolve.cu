@@ -1523,8 +1523,9 @@ void build_next(hsolve_handle* h, FLevel& FL, const real* arena, std::unique_ptr
 
 template <typename real>
 void factor_impl(hsolve_handle* h, double eps) {
-  // a merged dense top must fit the substitution sweeps' shared-memory slot
-  // vectors and, for a general matrix, the LU panel's thread-block cluster
+  // the interface's limit of a merged dense top: a slot vector of the sweeps in
+  // shared memory (the top's own kernels stream it in chunks and would take
+  // more) and, for a general matrix, the LU panel's thread-block cluster
   int64_t top_max = Launch<real>::apply_max_m();
   if (!h->symmetric) top_max = std::min<int64_t>(top_max, Launch<real>::lu_top_max());
   if (h->opts.top_size > top_max)

@@ -9,9 +9,9 @@
 // larger SPD ones and the shared helpers.
 //
 // Matrices are column-major.  `real` is the storage/compute type of the
-// factorization (double in float64 mode, float in the mixed modes); squared
-// column norms of the rank-revealing QR and its rank decision are always
-// accumulated in double.  The factor of A_ss and A_ss^{-1} live in shared
+// factorization (double in float64 mode, float in the mixed modes); the squared
+// column norms of the rank-revealing QR are accumulated in it, and its rank
+// decision is made in double.  The factor of A_ss and A_ss^{-1} live in shared
 // memory when they fit (the host sizes the dynamic shared memory per class);
 // everything else is in a per-cluster global workspace that stays in L2.
 #include <cfloat>
@@ -499,104 +499,79 @@ __device__ int cta_min_i(int v, int* red) {
   return r;
 }
 
-__device__ double cta_sum_d(double v, double* red) {
-  v = warp_sum(v);
-  if (lane_id() == 0) red[warp_id()] = v;
-  __syncthreads();
-  double r = 0;
-  for (int w = 0; w < num_warps(); w++) r += red[w];
-  __syncthreads();
-  return r;
-}
-
 // Householder QR of the m x c matrix G (in place).  Element (i, q) sits at
 // G[i * ldg + q] when RowMajor (one thread per column then reads coalesced
-// across a warp), else at G[i + q * ldg].  With `pivot`, columns are pivoted
-// by largest remaining norm (recomputed every step, near-ties to the lowest
-// original index, orig[] tracks original indices), stopping at
-// |r_jj| <= eps |r_11| (eps > 0), at |r_jj| <= floor (rounding noise of a
-// block that is zero in exact arithmetic), at an all-zero remainder or at
-// kmax steps.  Householder vectors stay in G (v_j in rows j..m of column j);
+// across a warp), else at G[i + q * ldg].  Columns are pivoted by largest
+// remaining norm (recomputed every step, near-ties to the lowest original
+// index, orig[] tracks original indices), stopping at |r_jj| <= eps |r_11|
+// (eps > 0), at |r_jj| <= floor (rounding noise of a block that is zero in
+// exact arithmetic), at an all-zero remainder or at kmax steps.  Householder vectors stay in G (v_j in rows j..m of column j);
 // tau[j] = 2 / v^T v.  vsh: m reals of shared memory.  Returns the number of
 // steps.
 template <typename real, bool RowMajor>
 __device__ int cta_householder_qr(int m, int c, real* G, int ldg, double* nrm2, double* orig,
-                                  real* tau, bool pivot, double eps, int kmax, double floor,
+                                  real* tau, double eps, int kmax, double floor,
                                   double* red_d, int* red_i, real* vsh, real* rsign = nullptr,
                                   const int* fpiv = nullptr) {
   auto at = [&](int i, int q) -> real& {
     return RowMajor ? G[(int64_t)i * ldg + q] : G[i + (int64_t)q * ldg];
   };
-  if (pivot) {
-    for (int q = threadIdx.x; q < c; q += blockDim.x) {
-      real s = 0;
-      for (int i = 0; i < m; i++) {
-        const real v = at(i, q);
-        s += v * v;
-      }
-      nrm2[q] = (double)s;
-      orig[q] = q;
+  for (int q = threadIdx.x; q < c; q += blockDim.x) {
+    real s = 0;
+    for (int i = 0; i < m; i++) {
+      const real v = at(i, q);
+      s += v * v;
     }
-    __syncthreads();
+    nrm2[q] = (double)s;
+    orig[q] = q;
   }
+  __syncthreads();
   double r11 = 0;
   int k = 0;
   const int steps = min(m, c);
   for (int j = 0; j < steps; j++) {
-    int q = j;
-    double r;
-    if (pivot) {
-      double mx = 0;
-      for (int t = j + threadIdx.x; t < c; t += blockDim.x) mx = fmax(mx, nrm2[t]);
-      mx = cta_max_d(mx, red_d);
-      if (mx == 0.0) break;
-      int best = INT_MAX;
-      if (fpiv) {
-        // a given pivot order (forced-rank factorization) replaces the search
-        best = j < kmax ? fpiv[j] : INT_MAX;
-      } else {
-        for (int t = j + threadIdx.x; t < c; t += blockDim.x)
-          if (nrm2[t] >= (1.0 - qr_tie_rtol<real>()) * mx) best = min(best, (int)orig[t]);
-        best = cta_min_i(best, red_i);
-      }
-      if (threadIdx.x == 0) red_i[blockDim.x] = -1;
-      __syncthreads();
-      for (int t = j + threadIdx.x; t < c; t += blockDim.x)
-        if ((int)orig[t] == best) red_i[blockDim.x] = t;
-      __syncthreads();
-      q = red_i[blockDim.x];
-      __syncthreads();
-      if (q < 0) break;  // the given pivot names no remaining column
-      r = sqrt(nrm2[q]);
-      if (j == 0) r11 = r;
-      if (r <= floor) break;
-      if (eps > 0.0 && r <= eps * r11) break;
-      if (j >= kmax) break;
-      if (q != j) {
-        for (int i = threadIdx.x; i < m; i += blockDim.x) {
-          real t = at(i, j);
-          at(i, j) = at(i, q);
-          at(i, q) = t;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          double t = nrm2[j];
-          nrm2[j] = nrm2[q];
-          nrm2[q] = t;
-          t = orig[j];
-          orig[j] = orig[q];
-          orig[q] = t;
-        }
-        __syncthreads();
-      }
+    double mx = 0;
+    for (int t = j + threadIdx.x; t < c; t += blockDim.x) mx = fmax(mx, nrm2[t]);
+    mx = cta_max_d(mx, red_d);
+    if (mx == 0.0) break;
+    int best = INT_MAX;
+    if (fpiv) {
+      // a given pivot order (forced-rank factorization) replaces the search
+      best = j < kmax ? fpiv[j] : INT_MAX;
     } else {
-      if (j >= kmax) break;
-      double s = 0;
-      for (int i = j + threadIdx.x; i < m; i += blockDim.x) {
-        double x = at(i, j);
-        s += x * x;
+      for (int t = j + threadIdx.x; t < c; t += blockDim.x)
+        if (nrm2[t] >= (1.0 - qr_tie_rtol<real>()) * mx) best = min(best, (int)orig[t]);
+      best = cta_min_i(best, red_i);
+    }
+    if (threadIdx.x == 0) red_i[blockDim.x] = -1;
+    __syncthreads();
+    for (int t = j + threadIdx.x; t < c; t += blockDim.x)
+      if ((int)orig[t] == best) red_i[blockDim.x] = t;
+    __syncthreads();
+    const int q = red_i[blockDim.x];
+    __syncthreads();
+    if (q < 0) break;  // the given pivot names no remaining column
+    const double r = sqrt(nrm2[q]);
+    if (j == 0) r11 = r;
+    if (r <= floor) break;
+    if (eps > 0.0 && r <= eps * r11) break;
+    if (j >= kmax) break;
+    if (q != j) {
+      for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        real t = at(i, j);
+        at(i, j) = at(i, q);
+        at(i, q) = t;
       }
-      r = sqrt(cta_sum_d(s, red_d));
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double t = nrm2[j];
+        nrm2[j] = nrm2[q];
+        nrm2[q] = t;
+        t = orig[j];
+        orig[j] = orig[q];
+        orig[q] = t;
+      }
+      __syncthreads();
     }
     // reflector v = x - beta e1, beta = -sign(x0) ||x||, tau = 2 / v^T v
     const double x0 = (double)at(j, j);
@@ -666,10 +641,9 @@ __device__ int cta_householder_qr(int m, int c, real* G, int ldg, double* nrm2, 
           }
         }
       }
-      if (pivot)
 #pragma unroll
-        for (int g = 0; g < CB; g++)
-          if (ok[g]) nrm2[t0 + g * nth] = (double)sq[g];
+      for (int g = 0; g < CB; g++)
+        if (ok[g]) nrm2[t0 + g * nth] = (double)sq[g];
     }
     __syncthreads();
     k = j + 1;
@@ -999,12 +973,12 @@ prep_kernel(const PrepTask* __restrict__ tasks, real* __restrict__ arena, real* 
     real* Yq = ysm ? W_B : Ysrc;
     const int ldY = ysm ? (m | 1) : m;
     if (ysm) cta_copy<real>(m, tk.l, Ysrc, m, Yq, ldY);
-    k = cta_householder_qr<real, false>(m, tk.l, Yq, ldY, nrm2, orig, tau, true, eps, kmax,
+    k = cta_householder_qr<real, false>(m, tk.l, Yq, ldY, nrm2, orig, tau, eps, kmax,
                                         noise_rtol * s_amax, red_d, red_i, vsh, rsign,
                                         fpiv ? fpiv + tk.pv : nullptr);
     cta_copy<real>(m, k, Yq, ldY, W_G, m);
   } else if (ncol > 0) {
-    k = cta_householder_qr<real, true>(m, ncol, W_G, ncol, nrm2, orig, tau, true, eps, kmax,
+    k = cta_householder_qr<real, true>(m, ncol, W_G, ncol, nrm2, orig, tau, eps, kmax,
                                        noise_rtol * s_amax, red_d, red_i, vsh, rsign,
                                        fpiv ? fpiv + tk.pv : nullptr);
   }

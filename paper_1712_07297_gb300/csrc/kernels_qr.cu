@@ -3,9 +3,9 @@
 //
 // The fill block G (m x c, c often in the thousands) is split by columns over
 // the CL CTAs of a thread-block cluster.  qr_reg_kernel keeps the columns in
-// registers for the whole factorization (clusters of up to 256 unknowns, fill
-// blocks that 8 CTAs hold); qr_cluster_kernel keeps them in shared memory
-// (larger ones).  Per step the CTAs agree on the pivot through distributed
+// registers for the whole factorization (float32 Cholesky path, clusters of up to
+// 256 unknowns, fill blocks that 16 CTAs hold); qr_cluster_kernel keeps them in
+// shared memory (the others).  Per step the CTAs agree on the pivot through distributed
 // shared memory: the largest remaining column norm over the cluster, then the
 // lowest original column index among the columns within the tie tolerance of
 // it (the tie rule of the single-CTA path); the reflector is formed from the
@@ -44,7 +44,7 @@ struct QrSmem {
   __host__ __device__ QrSmem(int ldsm, int cc, int sz) {
     G = 0;
     nrm = G + al((size_t)ldsm * cc * sz);
-    oidx = nrm + al((size_t)cc * sizeof(double));
+    oidx = nrm + al((size_t)cc * sizeof(double));  // (float32 norms use half of it)
     vloc = oidx + al((size_t)cc * sizeof(int));
     total = vloc + al((size_t)ldsm * sz);
   }
@@ -179,7 +179,8 @@ qr_cluster_kernel(const PrepTask* __restrict__ tasks, const int* __restrict__ or
   }
   __syncthreads();
   // squared norms in the working precision (float64 arithmetic per element
-  // would bound the float32 path by the float64 rate); compared in float64
+  // would bound the float32 path by the float64 rate), compared in it with
+  // thresholds that keep the float64 decisions (NormKey)
   for (int t = threadIdx.x; t < nloc; t += blockDim.x) {
     real s = 0;
     for (int i = 0; i < m; i++) {
