@@ -1,6 +1,7 @@
 // Internal declarations shared by the library's translation units.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <mutex>
 #include <cstddef>
@@ -118,8 +119,8 @@ __host__ __device__ __forceinline__ void householder_scalars(float r2, float x0,
   const float s = r2 > 0x1p100f ? 0x1p-40f : (r2 < 0x1p-80f ? 0x1p40f : 1.f);
   const float r2s = r2 * s * s, x0s = x0 * s;
   const float r = sqrtf(r2s);
-  if (!(r > 0.f)) {
-    *head = x0;
+  if (!(r > 0.f && r < HUGE_VALF)) {  // no column, or a norm beyond the floats
+    *head = x0 >= 0.f ? x0 + r : x0 - r;
     *tau = 0.f;
     return;
   }
@@ -140,6 +141,7 @@ __host__ __device__ __forceinline__ void householder_scalars(float r2, float x0,
 // largest, M.  The smallest float that is not below (1 - 1e-5) M, the product in
 // a pair of floats: a float32 norm compares with it as with the float64 product.
 __host__ __device__ __forceinline__ float tie_band(float M) {
+  if (!(M < HUGE_VALF)) return M;
   constexpr double c = 1.0 - 1e-5;
   constexpr float ch = (float)c, cl = (float)(c - (double)(float)c);
   const float p = M * ch;

@@ -73,10 +73,13 @@ def test_reflector_scalars(run, lo, hi):
         assert (got[fin] != w32[fin])[normal].mean() < 1e-4
 
 
-def test_no_column(run):
-    z = np.zeros(2, np.float32)
-    head, tau, _ = run(z, z)
-    assert not head.any() and not tau.any()
+def test_no_column_and_overflow(run):
+    # as the float64 form: no reflector
+    r2 = np.array([0, 0, np.inf, np.inf], np.float32)
+    x0 = np.array([0, 0, 3, -3], np.float32)
+    head, tau, band = run(r2, x0)
+    assert head.tolist() == [0, 0, np.inf, -np.inf] and not tau.any()
+    assert band.tolist() == [0, 0, np.inf, np.inf]
 
 
 @pytest.mark.parametrize("lo,hi", [(-90, 127.9)])
