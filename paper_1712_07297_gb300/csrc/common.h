@@ -5,7 +5,6 @@
 #include <cstdint>
 #include <mutex>
 #include <cstddef>
-#include <cstring>
 #include <string>
 #include <vector>
 
@@ -138,22 +137,20 @@ __host__ __device__ __forceinline__ void householder_scalars(float r2, float x0,
 
 // Near-ties of the float32 pivot search: squared norms carry ~1e-7 relative
 // rounding, so ties of exact arithmetic are recognised within 1e-5 of the
-// largest, M.  The smallest float that is not below (1 - 1e-5) M, the product in
-// a pair of floats: a float32 norm compares with it as with the float64 product.
+// largest, M.  The smallest float that is not below (1 - 1e-5) M, with the factor
+// in a pair of floats and one rounding, upwards: a float32 norm compares with it
+// as with the float64 product.
 __host__ __device__ __forceinline__ float tie_band(float M) {
-  if (!(M < HUGE_VALF)) return M;
   constexpr double c = 1.0 - 1e-5;
   constexpr float ch = (float)c, cl = (float)(c - (double)(float)c);
-  const float p = M * ch;
-  const float lo = fmaf(M, cl, fmaf(M, ch, -p));  // (1 - 1e-5) M = p + lo
-  float b = p + lo;
-  if (lo - (b - p) > 0.f) {  // rounded down: one float up
-    unsigned u;
-    memcpy(&u, &b, sizeof(u));
-    u++;
-    memcpy(&b, &u, sizeof(u));
-  }
-  return b;
+  if (!(M < HUGE_VALF)) return M;
+#ifdef __CUDA_ARCH__
+  return __fmaf_ru(M, ch, M * cl);
+#else
+  const double v = (double)M * ch + (double)M * cl;
+  const float b = (float)v;
+  return (double)b < v ? nextafterf(b, HUGE_VALF) : b;
+#endif
 }
 #endif
 

@@ -1,6 +1,6 @@
-"""The float32 scalars of the pivoted QRs, on the host, against float64: the head and
-tau of a reflector are the float64 ones rounded once (within 0.501 ulp) wherever that
-is a finite float, columns of norms up to the square root of the largest float
+"""The float32 scalars of the pivoted QRs, on the host and on the device, against
+float64: the head and tau of a reflector are the float64 ones rounded once (within
+0.501 ulp) wherever that is a finite float, columns of norms up to the square root of the largest float
 included, and the near-tie threshold is the smallest float not below the float64
 product."""
 import ctypes as C
@@ -16,6 +16,17 @@ PKG = os.path.join(ROOT, "paper_1712_07297_gb300")
 
 SOURCE = """
 #include "common.h"
+__global__ void kernel(long n, const float* r2, const float* x0, float* out) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
+       i += gridDim.x * (long)blockDim.x) {
+    hs::householder_scalars(r2[i], x0[i], out + i, out + n + i);
+    out[2 * n + i] = hs::tie_band(r2[i]);
+  }
+}
+extern "C" int run_device(long n, const float* r2, const float* x0, float* out) {
+  kernel<<<64, 256>>>(n, r2, x0, out);
+  return (int)cudaDeviceSynchronize();
+}
 extern "C" void run(long n, const float* r2, const float* x0, float* head, float* tau,
                     float* band) {
   for (long i = 0; i < n; i++) {
@@ -27,7 +38,7 @@ extern "C" void run(long n, const float* r2, const float* x0, float* head, float
 
 
 @pytest.fixture(scope="module")
-def run(tmp_path_factory):
+def lib(tmp_path_factory):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     d = tmp_path_factory.mktemp("scalars")
     (d / "s.cu").write_text(SOURCE)
@@ -35,15 +46,29 @@ def run(tmp_path_factory):
                     "arch=compute_103a,code=sm_103a", "--expt-relaxed-constexpr",
                     "-I" + os.path.join(PKG, "csrc"), "-I" + os.path.join(ROOT, "include"),
                     "-o", str(d / "s.so"), str(d / "s.cu")], check=True)
-    fn = C.CDLL(str(d / "s.so"), mode=os.RTLD_LAZY).run
-    fn.argtypes = [C.c_long] + [C.c_void_p] * 5
+    return C.CDLL(str(d / "s.so"), mode=os.RTLD_LAZY)
 
-    def call(r2, x0):
+
+@pytest.fixture(scope="module", params=["host", pytest.param("device", marks=pytest.mark.gpu)])
+def run(request, lib):
+    def host(r2, x0):
+        lib.run.argtypes = [C.c_long] + [C.c_void_p] * 5
         out = [np.empty_like(r2) for _ in range(3)]
-        fn(len(r2), r2.ctypes.data, x0.ctypes.data, *[o.ctypes.data for o in out])
+        lib.run(len(r2), r2.ctypes.data, x0.ctypes.data, *[o.ctypes.data for o in out])
         return out
 
-    return call
+    def device(r2, x0):
+        import torch
+        if not torch.cuda.is_available():
+            pytest.skip("no CUDA device")
+        lib.run_device.argtypes = [C.c_long] + [C.c_void_p] * 3
+        a, b = torch.from_numpy(r2).cuda(), torch.from_numpy(x0).cuda()
+        out = torch.empty(3 * len(r2), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        assert lib.run_device(len(r2), a.data_ptr(), b.data_ptr(), out.data_ptr()) == 0
+        return list(out.cpu().numpy().reshape(3, -1))
+
+    return host if request.param == "host" else device
 
 
 def _columns(lo, hi, n=400_000):
@@ -65,7 +90,8 @@ def test_reflector_scalars(run, lo, hi):
             w32 = want.astype(np.float32)
         fin = np.isfinite(w32)
         assert np.array_equal(np.isinf(got), ~fin)
-        err = np.abs(got[fin].astype(np.float64) - want[fin]) / np.spacing(np.abs(w32[fin])).astype(np.float64)
+        ulp = np.spacing(np.abs(w32[fin])).astype(np.float64)
+        err = np.abs(got[fin].astype(np.float64) - want[fin]) / ulp
         # (a tau below the normal floats is rounded twice: once more when scaled)
         bar = np.where(np.abs(want[fin]) < 2.0 ** -126, 0.7505, 0.501)
         assert (err <= bar).all(), (lo, hi, (err - bar).max())
