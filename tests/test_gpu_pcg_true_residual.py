@@ -1,4 +1,4 @@
-"""PCG ends on its recursive residual; the call is judged by the true one, b - A x.
+"""PCG ends on its recursive residual; the call reports the true one, b - A x.
 A tolerance that the true residual can meet must be met: near the rounding level of
 b - A x the two differ by more than the step between iterations leaves, and the
 solve has to go on from the true residual instead of giving up.
